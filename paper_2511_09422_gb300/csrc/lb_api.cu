@@ -31,6 +31,7 @@ struct lb_handle {
     lbk::StepRec *rec = nullptr;          // the step kernel's record of this lattice
     unsigned long long *counter = nullptr;  // the step kernel's work counters (2)
     long long nitems = 0;                   // work items of one step
+    int batch_segh = 0;          // segment rows in the steps of a batch (its own calls keep K.segh)
     int red_parts = 0;           // partial slots: one per warp of the largest capped MODE_REDUCE grid
     bool half = false;           // some populations stored in half precision
     // kernel instantiation: 0 FP32 D2Q9, 1 FP16 D2Q9, 2 FP32 with D2Q5 f and l, 3 FP16 f, g, l with FP32 h
@@ -153,6 +154,37 @@ static std::string check_params(const lb_grid *g, const lb_params *p)
     return "";
 }
 
+// Rows of an inner segment: the height, at most max_rows, of the lowest estimated
+// step time when it cuts the work into items(h) items.  An item runs h + 3 rows
+// one after another (its own, and the fill of the rings).  The warps of the wave
+// take the items in rounds of W; a row takes longer the more warps share a
+// scheduler (1.45 us with one, 2.1 us with two FP32 warps), and with many rounds
+// the last one is only partly filled.  Measured for heights 1 .. 16 (us per step):
+//   film 64 x 256: 9.2 at 2 rows, 17.0 at 8;   512 x 256: 15.1 at 4, 23.5 at 8;
+//   256^2: 11.4 at 2, 17.5 at 8;   512^2: 25.5 at 8, 28.5 at 4, 32.2 at 3;
+//   1037 x 771 (D2Q5): 61.6 at 12, 64.0 at 8, 72.2 at 10;   1024^2: 87.8 at 10, 95.1 at 12.
+// The estimate picks the best or the second best height in each of them.
+template <class Items>
+static int best_segment_rows(int kind, int max_rows, Items items)
+{
+    const long long W = with_storage(kind, [](auto ps) {
+        return 152LL * lbk::step_min_blocks<decltype(ps)>() * lbk::step_warps<decltype(ps)>();
+    });
+    int best = 1;
+    double least = 0.0;
+    for (int h = 1; h <= max_rows; h++) {
+        const long long n = items(h);
+        const double waves = (double)n / (double)W, rounds = waves <= 8.0 ? std::ceil(waves) : waves + 0.5;
+        const long long per_scheduler = ((n < W ? n : W) + 607) / 608;
+        const double cost = rounds * (h + 3) * (1.0 + 0.45 * (double)(per_scheduler - 1));
+        if (h == 1 || cost < least) {
+            least = cost;
+            best = h;
+        }
+    }
+    return best;
+}
+
 static Consts make_consts(const lb_grid *g, const lb_params *p)
 {
     Consts K;
@@ -192,24 +224,11 @@ static Consts make_consts(const lb_grid *g, const lb_params *p)
     K.gx = (real)p->gx; K.gy = (real)p->gy;
     K.expand = (real)(1.0 - p->rho_s / p->rho_l);
     K.fs_mod = p->fs_modulated_st ? 1 : 0;
-    K.segh = (p->pop_storage != LB_STORAGE_F32 || p->lattice_fl == LB_LATTICE_D2Q5) ? LB_SEGH_ALT : LB_SEGH;
-    // Shorter segments where the lattice gives the persistent wave of W warps too
-    // few work items.  A work item costs about segh + 3 rows (its rows plus the
-    // fill and copy prologue); the warps share the items dynamically, so a step
-    // takes about items (segh + 3) / W plus one item, the last one started.  The
-    // height of the default and the shorter candidates (8 rows at least) that
-    // minimises it.
     {
-        const long long W = with_storage(kind_of(p), [](auto ps) {
-            return 152LL * lbk::step_min_blocks<decltype(ps)>() * lbk::step_warps<decltype(ps)>();
-        });
+        const int kind = kind_of(p);
         const long long nstrip = (g->nx + LB_TX - 1) / LB_TX;
-        auto cost = [&](int h) { return (double)(nstrip * lbk::strip_segments(g->ny, h)) * (h + 3) / (double)W + (h + 3); };
-        const int cand[] = {24, 16, 12, 8};
-        int best = K.segh;
-        for (int c : cand)
-            if (c < K.segh && cost(c) < cost(best)) best = c;
-        K.segh = best;
+        K.segh = best_segment_rows(kind, kind == 0 ? LB_SEGH : LB_SEGH_ALT,
+                                   [&](int h) { return nstrip * lbk::strip_segments(g->ny, h); });
     }
     K.qfl = p->lattice_fl == LB_LATTICE_D2Q5 ? 5 : 9;
     K.divu = p->divu_mode;
@@ -272,11 +291,13 @@ static int flat_blocks(long long n, int threads)
     return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
 }
 
-// Record of lattice h for the step kernel, its work items numbered from item0;
+// Record of lattice h for the step kernel, with inner segments of segh rows, its
+// work items numbered from item0;
 // returns the number of items.
-static long long fill_record(const lb_handle *h, lbk::StepRec &r, long long item0)
+static long long fill_record(const lb_handle *h, lbk::StepRec &r, long long item0, int segh)
 {
     r.K = h->K;
+    r.K.segh = segh;
     for (int p = 0; p < 2; p++) {
         r.B[p].pin = h->pops[p];
         r.B[p].pout = h->pops[1 - p];
@@ -287,11 +308,13 @@ static long long fill_record(const lb_handle *h, lbk::StepRec &r, long long item
     }
     r.nstrip = (h->K.nx + LB_TX - 1) / LB_TX;
     r.item0 = item0;
-    return (long long)r.nstrip * lbk::strip_segments(h->K.ny, h->K.segh);
+    return (long long)r.nstrip * lbk::strip_segments(h->K.ny, segh);
 }
 
 // One step of ninst lattices (records rec, nitems work items in all) from buffer
-// `parity`: a persistent launch of at most one wave of resident blocks.
+// `parity`: a persistent launch of at most one wave of resident blocks, with
+// programmatic dependent launch, so that the blocks of the next step start while
+// this one's last ones finish (step_begin).
 template <class PS>
 static cudaError_t launch_step_as(const lbk::StepRec *rec, int ninst, long long nitems, int parity,
                                   unsigned long long *counter, cudaStream_t st)
@@ -307,9 +330,17 @@ static cudaError_t launch_step_as(const lbk::StepRec *rec, int ninst, long long 
     }
     // one persistent wave: as many blocks per SM as the rings of PS allow
     const long long wave = 152LL * lbk::step_min_blocks<PS>(), need = (nitems + sw - 1) / sw;
-    const unsigned grid = (unsigned)(need < wave ? (need < 1 ? 1 : need) : wave);
-    lbk::lb_step_kernel<PS><<<grid, dim3(32, sw, 1), smem, st>>>(rec, ninst, nitems, parity, counter);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(need < wave ? (need < 1 ? 1 : need) : wave));
+    cfg.blockDim = dim3(32, sw, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, lbk::lb_step_kernel<PS>, rec, ninst, nitems, parity, counter);
 }
 
 static cudaError_t launch_step(const lbk::StepRec *rec, int ninst, long long nitems, int parity,
@@ -332,7 +363,7 @@ static lb_status launch_reduce(lb_handle *h, double out[lbk::NRED])
     B.status = h->status;
     launch_strip<lbk::MODE_REDUCE>(K, B, h->stream, h->kind, h->partials);
     CK(h, cudaGetLastError());
-    // the warps of this launch's grid (the segment height, and so the grid, can change with lb_batch_tune)
+    // the warps of this launch's grid
     const int nparts = (int)with_storage(h->kind, [&](auto ps) { return reduce_blocks<decltype(ps)>(K); }) * LB_SW;
     lbk::lb_reduce_final_kernel<<<1, lbk::RED_THREADS, 0, h->stream>>>(h->partials, nparts, h->red_out);
     CK(h, cudaGetLastError());
@@ -408,7 +439,7 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
         cudaError_t me = cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream);
         if (me == cudaSuccess) me = cudaMemsetAsync(h->counter, 0, 2 * sizeof(unsigned long long), h->stream);
         lbk::StepRec rec;
-        h->nitems = fill_record(h, rec, 0);
+        h->nitems = fill_record(h, rec, 0, h->K.segh);
         if (me == cudaSuccess) me = cudaMemcpyAsync(h->rec, &rec, sizeof(rec), cudaMemcpyHostToDevice, h->stream);
         if (me != cudaSuccess) { st = cuda_fail(h, me, "step record"); break; }
         for (int k = 0; k < 5; k++) {
@@ -907,7 +938,7 @@ static int size_class(const lb_handle *h) { return h->K.ny < 192 ? 0 : (h->K.ny 
 static lb_status upload_instances(lb_batch *b)
 {
     long long item = 0;
-    for (size_t i = 0; i < b->h.size(); i++) item += fill_record(b->h[i], b->inst[i], item);
+    for (size_t i = 0; i < b->h.size(); i++) item += fill_record(b->h[i], b->inst[i], item, b->h[i]->batch_segh);
     b->nitems = item;
     BCK(b, cudaMemcpy(b->d_inst, b->inst.data(), sizeof(lbk::StepRec) * b->inst.size(), cudaMemcpyHostToDevice));
     drop_graphs(b);
@@ -941,6 +972,14 @@ extern "C" lb_status lb_batch_create(int n, const lb_grid *grids, const lb_param
                                                           ": all instances must use the same pop_storage and lattice_fl");
         }
     }
+    // the instances share the wave: segment heights for the work of the whole batch
+    const int segh = best_segment_rows(b->h[0]->kind, LB_SEGH_BATCH, [&](int rows) {
+        long long items = 0;
+        for (const lb_handle *h : b->h)
+            items += (long long)((h->K.nx + LB_TX - 1) / LB_TX) * lbk::strip_segments(h->K.ny, rows);
+        return items;
+    });
+    for (lb_handle *h : b->h) h->batch_segh = segh;
     b->inst.resize(n);
     lb_status s = LB_OK;
     cudaError_t e = cudaMalloc((void **)&b->d_inst, sizeof(lbk::StepRec) * n);
@@ -1033,7 +1072,7 @@ extern "C" lb_status lb_batch_tune(lb_batch *b, int trials, int seg_rows[3])
         int best = 0;
         for (int k = 0; k < 6 && st == LB_OK; k++) {
             for (lb_handle *h : b->h)
-                if (size_class(h) == c) h->K.segh = cand[k];
+                if (size_class(h) == c) h->batch_segh = cand[k];
             st = upload_instances(b);
             // trial launches read the current buffer and write the other one, which the
             // next real step overwrites: the state does not move
@@ -1051,7 +1090,7 @@ extern "C" lb_status lb_batch_tune(lb_batch *b, int trials, int seg_rows[3])
             }
         }
         for (lb_handle *h : b->h)
-            if (size_class(h) == c) h->K.segh = best;
+            if (size_class(h) == c) h->batch_segh = best;
         best_all[c] = best;
     }
     cudaEventDestroy(e0);
