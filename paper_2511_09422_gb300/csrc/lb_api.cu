@@ -26,7 +26,7 @@ struct lb_handle {
     float *aux[2] = {nullptr, nullptr};
     float *fields = nullptr;     // 7 planes
     double *partials = nullptr;  // reduction partials, red_parts * NRED
-    double *red_out = nullptr;   // NRED doubles on the device
+    double *red_out = nullptr;   // NRED sums and the status word on the device
     unsigned *status = nullptr;
     lbk::StepRec *rec = nullptr;          // the step kernel's record of this lattice
     unsigned long long *counter = nullptr;  // the step kernel's work counters (2)
@@ -263,6 +263,23 @@ static int carveout_for(int blocks, size_t smem)
     return pct > 100 ? 100 : pct;
 }
 
+// Launch with programmatic dependent launch (the kernel calls sweep_begin).
+template <class... P, class... A>
+static cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 template <int MODE, class PS>
 static void launch_strip_as(const Consts &K, const lbk::Buffers &B, cudaStream_t st, double *partials)
 {
@@ -275,7 +292,7 @@ static void launch_strip_as(const Consts &K, const lbk::Buffers &B, cudaStream_t
         opted = true;
     }
     const unsigned grid = MODE == lbk::MODE_REDUCE ? reduce_blocks<PS>(K) : strip_blocks(K);
-    lbk::lb_strip_kernel<MODE, PS><<<grid, dim3(32, LB_SW, 1), smem, st>>>(K, B, partials);
+    launch_dependent(lbk::lb_strip_kernel<MODE, PS>, grid, dim3(32, LB_SW, 1), smem, st, K, B, partials);
 }
 
 template <int MODE>
@@ -303,7 +320,6 @@ static long long fill_record(const lb_handle *h, lbk::StepRec &r, long long item
         r.B[p].pout = h->pops[1 - p];
         r.B[p].ain = h->aux[p];
         r.B[p].aout = h->aux[1 - p];
-        r.B[p].fields = nullptr;
         r.B[p].status = h->status;
     }
     r.nstrip = (h->K.nx + LB_TX - 1) / LB_TX;
@@ -312,9 +328,7 @@ static long long fill_record(const lb_handle *h, lbk::StepRec &r, long long item
 }
 
 // One step of ninst lattices (records rec, nitems work items in all) from buffer
-// `parity`: a persistent launch of at most one wave of resident blocks, with
-// programmatic dependent launch, so that the blocks of the next step start while
-// this one's last ones finish (step_begin).
+// `parity`: a persistent launch of at most one wave of resident blocks.
 template <class PS>
 static cudaError_t launch_step_as(const lbk::StepRec *rec, int ninst, long long nitems, int parity,
                                   unsigned long long *counter, cudaStream_t st)
@@ -330,17 +344,8 @@ static cudaError_t launch_step_as(const lbk::StepRec *rec, int ninst, long long 
     }
     // one persistent wave: as many blocks per SM as the rings of PS allow
     const long long wave = 152LL * lbk::step_min_blocks<PS>(), need = (nitems + sw - 1) / sw;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(need < wave ? (need < 1 ? 1 : need) : wave));
-    cfg.blockDim = dim3(32, sw, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lbk::lb_step_kernel<PS>, rec, ninst, nitems, parity, counter);
+    const unsigned grid = (unsigned)(need < wave ? (need < 1 ? 1 : need) : wave);
+    return launch_dependent(lbk::lb_step_kernel<PS>, grid, dim3(32, sw, 1), smem, st, rec, ninst, nitems, parity, counter);
 }
 
 static cudaError_t launch_step(const lbk::StepRec *rec, int ninst, long long nitems, int parity,
@@ -351,23 +356,21 @@ static cudaError_t launch_step(const lbk::StepRec *rec, int ninst, long long nit
     });
 }
 
-static lb_status launch_reduce(lb_handle *h, double out[lbk::NRED])
+// The diagnostics sums and, in out[NRED], the status word (0: no non-finite value).
+static lb_status launch_reduce(lb_handle *h, double out[lbk::NRED + 1])
 {
     const Consts &K = h->K;
-    lbk::Buffers B;
+    lbk::Buffers B = {};
     B.pin = h->pops[h->cur];
-    B.pout = nullptr;
     B.ain = h->aux[h->cur];
-    B.aout = nullptr;
-    B.fields = nullptr;
     B.status = h->status;
     launch_strip<lbk::MODE_REDUCE>(K, B, h->stream, h->kind, h->partials);
     CK(h, cudaGetLastError());
     // the warps of this launch's grid
     const int nparts = (int)with_storage(h->kind, [&](auto ps) { return reduce_blocks<decltype(ps)>(K); }) * LB_SW;
-    lbk::lb_reduce_final_kernel<<<1, lbk::RED_THREADS, 0, h->stream>>>(h->partials, nparts, h->red_out);
-    CK(h, cudaGetLastError());
-    CK(h, cudaMemcpyAsync(out, h->red_out, sizeof(double) * lbk::NRED, cudaMemcpyDeviceToHost, h->stream));
+    CK(h, launch_dependent(lbk::lb_reduce_final_kernel, 1, dim3(lbk::FINAL_THREADS), 0, h->stream, h->partials, nparts,
+                           h->status, h->red_out));
+    CK(h, cudaMemcpyAsync(out, h->red_out, sizeof(double) * (lbk::NRED + 1), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     return LB_OK;
 }
@@ -418,7 +421,7 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
     for (int k = 0; k < 2 && e == cudaSuccess; k++) e = alloc((void **)&h->aux[k], lbk::NAUX * plane_b);
     if (e == cudaSuccess) e = alloc((void **)&h->fields, 7 * plane_b);
     if (e == cudaSuccess) e = alloc((void **)&h->partials, sizeof(double) * lbk::NRED * h->red_parts);
-    if (e == cudaSuccess) e = alloc((void **)&h->red_out, sizeof(double) * lbk::NRED);
+    if (e == cudaSuccess) e = alloc((void **)&h->red_out, sizeof(double) * (lbk::NRED + 1));
     if (e == cudaSuccess) e = alloc((void **)&h->status, sizeof(unsigned));
     if (e == cudaSuccess) e = alloc((void **)&h->rec, sizeof(lbk::StepRec));
     if (e == cudaSuccess) e = alloc((void **)&h->counter, 2 * sizeof(unsigned long long));
@@ -474,7 +477,7 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
         }
         if (ce != cudaSuccess) { st = cuda_fail(h, ce, "init kernels"); break; }
         h->cur = 0;
-        double r[lbk::NRED];
+        double r[lbk::NRED + 1];
         st = launch_reduce(h, r);
         if (st != LB_OK) break;
         h->V0 = r[4];
@@ -599,28 +602,41 @@ extern "C" lb_status lb_steps_taken(lb_handle *h, long *out)
     return LB_OK;
 }
 
+// Whether a kernel on the current device may use p in place: an aligned array in
+// this device's own memory.
+static bool own_memory(const float *p)
+{
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (((uintptr_t)p & 3) || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 extern "C" lb_status lb_get_fields(lb_handle *h, float *phi, float *T, float *fs, float *C, float *ux, float *uy,
                                    float *p, int on_device)
 {
     if (!h) return LB_ERR_INVALID_ARG;
     if (h->sticky != LB_OK) return h->sticky;
     const Consts &K = h->K;
-    lbk::Buffers B;
+    // outputs in this device's memory are written in place, others by way of the 7-plane field buffer (dense)
+    float *dst[7] = {phi, T, fs, C, ux, uy, p};
+    const size_t n = (size_t)K.nx * K.ny;
+    bool in_place[7];
+    for (int k = 0; k < 7; k++) in_place[k] = dst[k] && on_device && own_memory(dst[k]);
+    lbk::Buffers B = {};
     B.pin = h->pops[h->cur];
-    B.pout = nullptr;
     B.ain = h->aux[h->cur];
-    B.aout = nullptr;
-    B.fields = h->fields;
     B.status = h->status;
+    for (int k = 0; k < 7; k++) B.out[k] = !dst[k] || in_place[k] ? dst[k] : h->fields + k * n;
+    B.out_pitch = K.nx;
     launch_strip<lbk::MODE_FIELDS>(K, B, h->stream, h->kind);
     CK(h, cudaGetLastError());
-    float *dst[7] = {phi, T, fs, C, ux, uy, p};
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    for (int k = 0; k < 7; k++) {
-        if (!dst[k]) continue;
-        CK(h, cudaMemcpy2DAsync(dst[k], sizeof(float) * K.nx, h->fields + (size_t)k * K.plane, sizeof(float) * K.pitch,
-                                sizeof(float) * K.nx, K.ny, kind, h->stream));
-    }
+    for (int k = 0; k < 7; k++)
+        if (dst[k] && !in_place[k]) CK(h, cudaMemcpyAsync(dst[k], B.out[k], sizeof(float) * n, kind, h->stream));
     if (!on_device) CK(h, cudaStreamSynchronize(h->stream));
     return LB_OK;
 }
@@ -668,12 +684,10 @@ extern "C" lb_status lb_reduce(lb_handle *h, double out[8])
 {
     if (!h || !out) return fail(h, LB_ERR_INVALID_ARG, "null argument");
     if (h->sticky != LB_OK) return h->sticky;
-    double r[lbk::NRED];
+    double r[lbk::NRED + 1];
     lb_status s = launch_reduce(h, r);
     if (s != LB_OK) return s;
-    unsigned status = 0;
-    CK(h, cudaMemcpyAsync(&status, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    const bool status = r[lbk::NRED] != 0.0;
     for (int k = 0; k < 6; k++) out[k] = r[k];
     out[6] = h->V0 > 0 ? r[3] / h->V0 : 0.0;
     out[7] = h->V0 > 0 ? r[4] / h->V0 : 0.0;
