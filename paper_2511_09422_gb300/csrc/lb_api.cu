@@ -33,7 +33,6 @@ struct lb_handle {
     long long nitems = 0;                   // work items of one step
     int batch_segh = 0;          // segment rows in the steps of a batch (its own calls keep K.segh)
     int red_parts = 0;           // partial slots: one per warp of the largest capped MODE_REDUCE grid
-    bool half = false;           // some populations stored in half precision
     // kernel instantiation: 0 FP32 D2Q9, 1 FP16 D2Q9, 2 FP32 with D2Q5 f and l, 3 FP16 f, g, l with FP32 h
     int kind = 0;
     size_t pop_bytes() const;
@@ -375,6 +374,46 @@ static lb_status launch_reduce(lb_handle *h, double out[lbk::NRED + 1])
     return LB_OK;
 }
 
+// Whether a kernel on the current device may use p in place: an aligned array in
+// this device's own memory.
+static bool own_memory(const float *p)
+{
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (((uintptr_t)p & 3) || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
+// The state of h from the given fields (phi, T, C, ux, uy, fs, p; null where not
+// given): arrays in this device's own memory are read in place, others come by way
+// of the 7-plane field buffer (dense).
+static cudaError_t set_state(lb_handle *h, const float *const src[7], bool on_device, int match_moment)
+{
+    const Consts &K = h->K;
+    const size_t n = (size_t)K.nx * K.ny;
+    const float *dev[7];
+    for (int k = 0; k < 7; k++) {
+        dev[k] = src[k];
+        if (!src[k] || (on_device && own_memory(src[k]))) continue;
+        float *d = h->fields + (size_t)k * n;
+        const cudaError_t e = cudaMemcpyAsync(d, src[k], sizeof(float) * n,
+                                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream);
+        if (e != cudaSuccess) return e;
+        dev[k] = d;
+    }
+    const lbk::InitFields F = {dev[0], dev[1], dev[2], dev[3], dev[4], dev[5], dev[6]};
+    const unsigned blocks = (unsigned)((long long)((K.nx + 31) / 32) * ((K.ny + lbk::INIT_ROWS - 1) / lbk::INIT_ROWS));
+    with_storage(h->kind, [&](auto ps) {
+        lbk::lb_init_kernel<decltype(ps)><<<blocks, dim3(32, lbk::INIT_ROWS), 0, h->stream>>>(
+            K, F, h->pops[h->cur], h->aux[h->cur], match_moment);
+        return 0;
+    });
+    return cudaGetLastError();
+}
+
 static void free_all(lb_handle *h)
 {
     void *ptrs[] = {h->pops[0], h->pops[1], h->aux[0], h->aux[1], h->fields, h->partials, h->red_out, h->status,
@@ -396,7 +435,6 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
     lb_handle *h = new lb_handle();
     h->grid = *grid;
     h->params = *params;
-    h->half = params->pop_storage != LB_STORAGE_F32;
     h->kind = kind_of(params);
     h->K = make_consts(grid, params);
     h->K.ghost_lo = ghost_lo;
@@ -406,7 +444,6 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
             return (size_t)lbk::halo_message_bytes<decltype(ps)>(grid->nx);
         });
     const Consts &K = h->K;
-    const long long n = (long long)grid->nx * grid->ny;
     const size_t plane_b = sizeof(float) * (size_t)K.plane;
     // every grid reduce_blocks can give (a capped wave of at most 6 blocks per SM)
     h->red_parts = 152 * 6 * LB_SW;
@@ -434,49 +471,20 @@ static lb_status create_handle(const lb_grid *grid, const lb_params *params, con
         return s;
     }
 
-    // initial fields on the device (the field buffer serves as staging)
-    const float *src[5] = {init->phi, init->T, init->C, init->ux, init->uy};
-    const float *dev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     lb_status st = LB_OK;
     do {
         cudaError_t me = cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream);
+        // planes that a D2Q5 step does not write are zero in both buffers
+        if (me == cudaSuccess && h->kind == 2) me = cudaMemsetAsync(h->pops[1], 0, h->pop_bytes(), h->stream);
         if (me == cudaSuccess) me = cudaMemsetAsync(h->counter, 0, 2 * sizeof(unsigned long long), h->stream);
         lbk::StepRec rec;
         h->nitems = fill_record(h, rec, 0, h->K.segh);
         if (me == cudaSuccess) me = cudaMemcpyAsync(h->rec, &rec, sizeof(rec), cudaMemcpyHostToDevice, h->stream);
         if (me != cudaSuccess) { st = cuda_fail(h, me, "step record"); break; }
-        for (int k = 0; k < 5; k++) {
-            if (!src[k]) continue;
-            float *d = h->fields + (size_t)k * K.plane;
-            cudaError_t ce = cudaMemcpyAsync(d, src[k], sizeof(float) * n,
-                                             init->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream);
-            if (ce != cudaSuccess) { st = cuda_fail(h, ce, "copy of the initial fields"); break; }
-            dev[k] = d;
-        }
-        if (st != LB_OK) break;
-        // equilibria in FP32: in the second population buffer, or for half storage
-        // in a temporary buffer freed once the first buffer holds the state
-        float *eq = h->pops[1], *eq_tmp = nullptr;
-        if (h->half) {
-            cudaError_t ae = cudaMalloc((void **)&eq_tmp, 36 * plane_b);
-            if (ae != cudaSuccess) { st = cuda_fail(h, ae, "cudaMalloc of the initial equilibria"); break; }
-            eq = eq_tmp;
-        }
-        lbk::lb_init_eq_kernel<<<flat_blocks(n, 256), 256, 0, h->stream>>>(K, dev[0], dev[1], dev[2], dev[3], dev[4],
-                                                                           nullptr, nullptr, eq, h->aux[0], 0);
-        with_storage(h->kind, [&](auto ps) {
-            lbk::lb_init_unstream_kernel<decltype(ps)><<<flat_blocks(n, 256), 256, 0, h->stream>>>(K, eq, h->aux[0],
-                                                                                                  h->pops[0]);
-            return 0;
-        });
-        cudaError_t ce = cudaGetLastError();
-        if (eq_tmp) {
-            cudaError_t fe = cudaStreamSynchronize(h->stream);
-            cudaFree(eq_tmp);
-            if (ce == cudaSuccess) ce = fe;
-        }
-        if (ce != cudaSuccess) { st = cuda_fail(h, ce, "init kernels"); break; }
         h->cur = 0;
+        const float *src[7] = {init->phi, init->T, init->C, init->ux, init->uy, nullptr, nullptr};
+        const cudaError_t ce = set_state(h, src, init->on_device != 0, 0);
+        if (ce != cudaSuccess) { st = cuda_fail(h, ce, "initial state"); break; }
         double r[lbk::NRED + 1];
         st = launch_reduce(h, r);
         if (st != LB_OK) break;
@@ -602,19 +610,6 @@ extern "C" lb_status lb_steps_taken(lb_handle *h, long *out)
     return LB_OK;
 }
 
-// Whether a kernel on the current device may use p in place: an aligned array in
-// this device's own memory.
-static bool own_memory(const float *p)
-{
-    cudaPointerAttributes a;
-    int dev = -1;
-    if (((uintptr_t)p & 3) || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
-}
-
 extern "C" lb_status lb_get_fields(lb_handle *h, float *phi, float *T, float *fs, float *C, float *ux, float *uy,
                                    float *p, int on_device)
 {
@@ -647,35 +642,8 @@ extern "C" lb_status lb_set_fields(lb_handle *h, const float *phi, const float *
     if (!h) return LB_ERR_INVALID_ARG;
     if (h->sticky != LB_OK) return h->sticky;
     if (!phi || !T || !C) return fail(h, LB_ERR_INVALID_ARG, "phi, T and C are required");
-    const Consts &K = h->K;
-    const size_t n = (size_t)K.nx * K.ny;
-    // the inputs go to the 7-plane fields buffer first (dense, as lb_create does), in
-    // the argument order phi, T, C, ux, uy, fs, p
     const float *src[7] = {phi, T, C, ux, uy, fs, p};
-    const float *dev[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    for (int k = 0; k < 7; k++) {
-        if (!src[k]) continue;
-        float *d = h->fields + (size_t)k * K.plane;
-        CK(h, cudaMemcpyAsync(d, src[k], sizeof(float) * n, kind, h->stream));
-        dev[k] = d;
-    }
-    const size_t plane_b = sizeof(float) * (size_t)K.plane;
-    float *eq = h->pops[1 - h->cur], *eq_tmp = nullptr;
-    if (h->half) {
-        CK(h, cudaMallocAsync((void **)&eq_tmp, 36 * plane_b, h->stream));
-        eq = eq_tmp;
-    }
-    lbk::lb_init_eq_kernel<<<flat_blocks((long long)n, 256), 256, 0, h->stream>>>(K, dev[0], dev[1], dev[2], dev[3],
-                                                                                 dev[4], dev[5], dev[6], eq,
-                                                                                 h->aux[h->cur], 1);
-    with_storage(h->kind, [&](auto ps) {
-        lbk::lb_init_unstream_kernel<decltype(ps)><<<flat_blocks((long long)n, 256), 256, 0, h->stream>>>(
-            K, eq, h->aux[h->cur], h->pops[h->cur]);
-        return 0;
-    });
-    CK(h, cudaGetLastError());
-    if (eq_tmp) CK(h, cudaFreeAsync(eq_tmp, h->stream));
+    CK(h, set_state(h, src, on_device != 0, 1));
     if (!on_device) CK(h, cudaStreamSynchronize(h->stream));
     return LB_OK;
 }

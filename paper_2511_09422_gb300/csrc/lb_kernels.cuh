@@ -1685,10 +1685,21 @@ __global__ void __launch_bounds__(32 * step_warps<PS>(), step_min_blocks<PS>()) 
 }
 
 // ---------------------------------------------------------------------------------------
-// Initialisation: equilibria of the initial fields (p = 0), written in natural
-// (post-streaming) layout to `eq`, h as deviations from w_i rr T (with the
-// latent reference for i = 0), and the lagged fields of a state at rest in time.
+// Initialisation: equilibria of the given fields in natural (post-streaming)
+// layout, h as deviations from w_i rr T (with the latent reference for i = 0), then
+// inverse streaming: the stored state is post-collision, so each is placed where
+// the next pull finds it, f, g and h as deviations from the references of the cell
+// that holds them; and the lagged fields of a state at rest in time.
+// One pass: a block forms the equilibria of its tile and of the cells around it
+// in shared memory (1.6 times its own cells at 32 x 4) and writes the tile's 45
+// planes.  Passing the 36 equilibria through global memory between two kernels took
+// 149 us at 1024^2.  Bound by its stores.
 // ---------------------------------------------------------------------------------------
+// Dense nx * ny inputs; ux, uy, fs and p may be null.
+struct InitFields {
+    const float *phi, *T, *C, *ux, *uy, *fs, *p;
+};
+
 // Velocity component v (dense nx * ny input) at (x + dx, y + dy), with the
 // ghost -u of row y beyond a no-slip wall.
 __device__ __forceinline__ real dense_u_nb(const Consts &K, const float *__restrict__ v, int x, int y, int dx, int dy)
@@ -1698,86 +1709,88 @@ __device__ __forceinline__ real dense_u_nb(const Consts &K, const float *__restr
     return v[(long long)yy * K.nx + xx];
 }
 
-// match_moment (re-initialisation from fields): when div u is the lagged
+constexpr int INIT_ROWS = 4;                             // rows of a tile, 32 columns each
+constexpr int INIT_W = 34, INIT_N = INIT_W * (INIT_ROWS + 2);  // columns and cells with the halo
+struct InitTile {
+    float eq[36][INIT_N], T[INIT_N], p[INIT_N];
+};
+
+// Equilibria of cell (x, y) into slot n of the tile; its lagged fields into aux if
+// `own`.  match_moment (re-initialisation from fields): when div u is the lagged
 // velocity divergence, the next step reads phi = sum f / (1 - div u / 2) with
 // div u the divergence of the installed velocity; the rest population is then
 // lowered by phi div u / 2 so that this reading returns the given phi.
-__global__ void lb_init_eq_kernel(const Consts K, const float *__restrict__ phi0, const float *__restrict__ T0,
-                                  const float *__restrict__ C0, const float *__restrict__ ux0,
-                                  const float *__restrict__ uy0, const float *__restrict__ fs0,
-                                  const float *__restrict__ p0, float *__restrict__ eq, float *__restrict__ aux,
-                                  int match_moment)
+__device__ __forceinline__ void init_equilibria(const Consts &K, const InitFields &F, int x, int y, InitTile &t, int n,
+                                                bool own, float *__restrict__ aux, int match_moment)
 {
-    const long long n = (long long)K.nx * K.ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / K.nx), x = (int)(k % K.nx);
-        const long long cell = (long long)y * K.pitch + x;
-        const real phi = phi0[k], T = T0[k], C = C0[k];
-        const real ux = ux0 ? ux0[k] : R(0.0), uy = uy0 ? uy0[k] : R(0.0);
-        real f0_shift = R(0.0);
-        if (match_moment && K.divu && ux0 && uy0) {
-            const real dudx = wgt(1) * (dense_u_nb(K, ux0, x, y, 1, 0) - dense_u_nb(K, ux0, x, y, -1, 0)) +
-                              wgt(5) * ((dense_u_nb(K, ux0, x, y, 1, 1) - dense_u_nb(K, ux0, x, y, -1, 1)) +
-                                        (dense_u_nb(K, ux0, x, y, 1, -1) - dense_u_nb(K, ux0, x, y, -1, -1)));
-            const real dvdy = wgt(2) * (dense_u_nb(K, uy0, x, y, 0, 1) - dense_u_nb(K, uy0, x, y, 0, -1)) +
-                              wgt(5) * ((dense_u_nb(K, uy0, x, y, 1, 1) - dense_u_nb(K, uy0, x, y, 1, -1)) +
-                                        (dense_u_nb(K, uy0, x, y, -1, 1) - dense_u_nb(K, uy0, x, y, -1, -1)));
-            f0_shift = -R(0.5) * phi * R(3.0) * (dudx + dvdy);
-        }
-        const real chi = clamp01(R(0.5) * (R(1.0) + phi));
-        real fs;
-        real e_sens;
-        if (fs0) {
-            // given solid fraction (clamped to [0, chi]): sensible enthalpy by the
-            // mixture rule of the volumetric heat capacities
-            fs = K.phase_change ? fminf(fmaxf(fs0[k], R(0.0)), chi) : R(0.0);
-            e_sens = T * (fs * K.rcp_s + (chi - fs) * K.rcp_l + (R(1.0) - chi) * K.rcp_g);
-        } else {
-            e_sens = forward_sensible(K, T, chi, fs);
-        }
-        const real rho = zeta(phi, fs, K.rho_l, K.rho_s, K.rho_g);
-        const real rhocp = zeta(phi, fs, K.rcp_l, K.rcp_s, K.rcp_g);
-        const real uu = ux * ux + uy * uy;
-        const real rcT = rhocp * T;
+    const long long k = (long long)y * K.nx + x;
+    const real phi = F.phi[k], T = F.T[k], C = F.C[k];
+    const real ux = F.ux ? F.ux[k] : R(0.0), uy = F.uy ? F.uy[k] : R(0.0);
+    real f0_shift = R(0.0);
+    if (match_moment && K.divu && F.ux && F.uy) {
+        const float *ux0 = F.ux, *uy0 = F.uy;
+        const real dudx = wgt(1) * (dense_u_nb(K, ux0, x, y, 1, 0) - dense_u_nb(K, ux0, x, y, -1, 0)) +
+                          wgt(5) * ((dense_u_nb(K, ux0, x, y, 1, 1) - dense_u_nb(K, ux0, x, y, -1, 1)) +
+                                    (dense_u_nb(K, ux0, x, y, 1, -1) - dense_u_nb(K, ux0, x, y, -1, -1)));
+        const real dvdy = wgt(2) * (dense_u_nb(K, uy0, x, y, 0, 1) - dense_u_nb(K, uy0, x, y, 0, -1)) +
+                          wgt(5) * ((dense_u_nb(K, uy0, x, y, 1, 1) - dense_u_nb(K, uy0, x, y, 1, -1)) +
+                                    (dense_u_nb(K, uy0, x, y, -1, 1) - dense_u_nb(K, uy0, x, y, -1, -1)));
+        f0_shift = -R(0.5) * phi * R(3.0) * (dudx + dvdy);
+    }
+    const real chi = clamp01(R(0.5) * (R(1.0) + phi));
+    real fs;
+    real e_sens;
+    if (F.fs) {
+        // given solid fraction (clamped to [0, chi]): sensible enthalpy by the
+        // mixture rule of the volumetric heat capacities
+        fs = K.phase_change ? fminf(fmaxf(F.fs[k], R(0.0)), chi) : R(0.0);
+        e_sens = T * (fs * K.rcp_s + (chi - fs) * K.rcp_l + (R(1.0) - chi) * K.rcp_g);
+    } else {
+        e_sens = forward_sensible(K, T, chi, fs);
+    }
+    const real rho = zeta(phi, fs, K.rho_l, K.rho_s, K.rho_g);
+    const real rhocp = zeta(phi, fs, K.rcp_l, K.rcp_s, K.rcp_g);
+    const real uu = ux * ux + uy * uy;
+    const real rcT = rhocp * T;
 #pragma unroll
-        for (int i = 0; i < 9; i++) {
-            const real cu = (real)cx(i) * ux + (real)cy(i) * uy;
-            const real si = wgt(i) * (R(3.0) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-            eq[(long long)(SET_F * 9 + i) * K.plane + cell] =
-                wfl_rt(K.qfl, i) * phi * (R(1.0) + R(3.0) * cu) + (i == 0 ? f0_shift : R(0.0));
-            eq[(long long)(SET_G * 9 + i) * K.plane + cell] = rho * si;
-            eq[(long long)(SET_L * 9 + i) * K.plane + cell] = wfl_rt(K.qfl, i) * C * (R(1.0) + R(3.0) * cu);
-            // h_0 - w_0 rr T - latent = e_sens - rr T - w_0 rho Cp T 3u.u/2;  h_i - w_i rr T = w_i rho Cp T (...)
-            eq[(long long)(SET_H * 9 + i) * K.plane + cell] =
-                i == 0 ? e_sens - K.rr * T - wgt(0) * rcT * R(1.5) * uu
-                       : wgt(i) * rcT * (R(3.0) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-        }
-        aux[AUX_FS * K.plane + cell] = fs;
-        aux[AUX_Q * K.plane + cell] = 0.0f;
-        aux[AUX_UX * K.plane + cell] = ux;
-        aux[AUX_UY * K.plane + cell] = uy;
-        aux[AUX_PHI * K.plane + cell] = phi;
-        aux[AUX_C * K.plane + cell] = C;
-        aux[AUX_P * K.plane + cell] = p0 ? p0[k] : 0.0f;
-        aux[AUX_S * K.plane + cell] = 0.0f;
-        aux[AUX_T * K.plane + cell] = T;
+    for (int i = 0; i < 9; i++) {
+        const real cu = (real)cx(i) * ux + (real)cy(i) * uy;
+        const real si = wgt(i) * (R(3.0) * cu + R(4.5) * cu * cu - R(1.5) * uu);
+        t.eq[SET_F * 9 + i][n] = wfl_rt(K.qfl, i) * phi * (R(1.0) + R(3.0) * cu) + (i == 0 ? f0_shift : R(0.0));
+        t.eq[SET_G * 9 + i][n] = rho * si;
+        t.eq[SET_L * 9 + i][n] = wfl_rt(K.qfl, i) * C * (R(1.0) + R(3.0) * cu);
+        // h_0 - w_0 rr T - latent = e_sens - rr T - w_0 rho Cp T 3u.u/2;  h_i - w_i rr T = w_i rho Cp T (...)
+        t.eq[SET_H * 9 + i][n] = i == 0 ? e_sens - K.rr * T - wgt(0) * rcT * R(1.5) * uu
+                                        : wgt(i) * rcT * (R(3.0) * cu + R(4.5) * cu * cu - R(1.5) * uu);
+    }
+    const real p = F.p ? F.p[k] : 0.0f;
+    t.T[n] = T;
+    t.p[n] = p;
+    if (own) {
+        const int cell = y * K.pitch + x;
+        plane_ptr(aux, AUX_FS, K)[cell] = fs;
+        plane_ptr(aux, AUX_Q, K)[cell] = 0.0f;
+        plane_ptr(aux, AUX_UX, K)[cell] = ux;
+        plane_ptr(aux, AUX_UY, K)[cell] = uy;
+        plane_ptr(aux, AUX_PHI, K)[cell] = phi;
+        plane_ptr(aux, AUX_C, K)[cell] = C;
+        plane_ptr(aux, AUX_P, K)[cell] = p;
+        plane_ptr(aux, AUX_S, K)[cell] = 0.0f;
+        plane_ptr(aux, AUX_T, K)[cell] = T;
     }
 }
 
-// Inverse streaming: the stored state is post-collision, so the initial
-// post-streaming populations `eq` are placed where the next pull finds them,
-// f, g and h as deviations from the references of the cell that holds them.
+// Inverse streaming of set S for cell (x, y), slot n of the tile.
 template <class PS, int S>
-__device__ __forceinline__ void unstream_set(const Consts &K, const float *__restrict__ eq,
-                                             const float *__restrict__ aux, float *__restrict__ pops, int x, int y,
-                                             long long cell, real phi_here, real T_here)
+__device__ __forceinline__ void unstream_set(const Consts &K, const InitTile &t, float *__restrict__ pops, int x, int y,
+                                             int n, int cell, real phi_here, real T_here)
 {
 #pragma unroll
     for (int i = 0; i < 9; i++) {
         const int yt = y + cy(i);
         real v;
         if (yt < 0 || yt >= K.ny) {
-            v = eq[(long long)(S * 9 + opp(i)) * K.plane + cell];
+            v = t.eq[S * 9 + opp(i)][n];
             if (S == SET_H) {
                 const bool bottom = yt < 0;
                 if ((bottom ? K.bc_bottom : K.bc_top) == WALL_DIRICHLET) {
@@ -1787,33 +1800,46 @@ __device__ __forceinline__ void unstream_set(const Consts &K, const float *__res
                 }
             }
         } else {
-            const int xt = wrapx(x + cx(i), K.nx);
-            const long long ct = (long long)yt * K.pitch + xt;
-            v = eq[(long long)(S * 9 + i) * K.plane + ct];
-            if (S == SET_H && i != 0) v += wgt(i) * K.rr * ((real)aux[AUX_T * K.plane + ct] - T_here);
-            if (S == SET_G && i != 0)
-                v += R(3.0) * wgt(i) * ((real)aux[AUX_P * K.plane + ct] - (real)aux[AUX_P * K.plane + cell]);
+            const int nt = n + cy(i) * INIT_W + cx(i);
+            v = t.eq[S * 9 + i][nt];
+            if (S == SET_H && i != 0) v += wgt(i) * K.rr * (t.T[nt] - T_here);
+            if (S == SET_G && i != 0) v += R(3.0) * wgt(i) * (t.p[nt] - t.p[n]);
         }
-        if (S == SET_F) v -= wfl_rt(K.qfl, i) * phi_here;
+        if (S == SET_F) {
+            const real w = wfl_rt(K.qfl, i);
+            v = i == 0 ? __fmaf_rn(-w, phi_here, v) : __fsub_rn(v, __fmul_rn(w, phi_here));
+        }
         set_plane<PS, S>(pops, i, K)[cell] = enc_pop<PS, S>(K, i, v);
     }
 }
 
 template <class PS>
-__global__ void lb_init_unstream_kernel(const Consts K, const float *__restrict__ eq, const float *__restrict__ aux,
-                                        float *__restrict__ pops)
+__global__ void __launch_bounds__(32 * INIT_ROWS) lb_init_kernel(const Consts K, const InitFields F,
+                                                                 float *__restrict__ pops, float *__restrict__ aux,
+                                                                 int match_moment)
 {
-    const long long n = (long long)K.nx * K.ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / K.nx), x = (int)(k % K.nx);
-        const long long cell = (long long)y * K.pitch + x;
-        const real phi_here = aux[AUX_PHI * K.plane + cell];
-        const real T_here = aux[AUX_T * K.plane + cell];
-        unstream_set<PS, SET_F>(K, eq, aux, pops, x, y, cell, phi_here, T_here);
-        unstream_set<PS, SET_G>(K, eq, aux, pops, x, y, cell, phi_here, T_here);
-        unstream_set<PS, SET_H>(K, eq, aux, pops, x, y, cell, phi_here, T_here);
-        unstream_set<PS, SET_L>(K, eq, aux, pops, x, y, cell, phi_here, T_here);
+    __shared__ InitTile t;
+    const int nbx = (K.nx + 31) / 32;
+    const int x0 = (int)(blockIdx.x % nbx) * 32, y0 = (int)(blockIdx.x / nbx) * INIT_ROWS;
+    for (int n = threadIdx.y * 32 + threadIdx.x; n < INIT_N; n += 32 * INIT_ROWS) {
+        const int ly = n / INIT_W - 1, lx = n % INIT_W - 1, y = y0 + ly;
+        if (y < 0 || y >= K.ny) continue;
+        // columns right of the lattice are its first ones; beyond the one a halo needs they are not read
+        const int c = x0 + lx;
+        if (c > K.nx) continue;
+        const int x = c < 0 ? K.nx - 1 : (c == K.nx ? 0 : c);
+        const bool own = lx >= 0 && lx < 32 && ly >= 0 && ly < INIT_ROWS && c < K.nx;
+        init_equilibria(K, F, x, y, t, n, own, aux, match_moment);
     }
+    __syncthreads();
+    const int x = x0 + (int)threadIdx.x, y = y0 + (int)threadIdx.y;
+    if (x >= K.nx || y >= K.ny) return;
+    const int n = ((int)threadIdx.y + 1) * INIT_W + (int)threadIdx.x + 1, cell = y * K.pitch + x;
+    const real phi_here = F.phi[(long long)y * K.nx + x], T_here = t.T[n];
+    unstream_set<PS, SET_F>(K, t, pops, x, y, n, cell, phi_here, T_here);
+    unstream_set<PS, SET_G>(K, t, pops, x, y, n, cell, phi_here, T_here);
+    unstream_set<PS, SET_H>(K, t, pops, x, y, n, cell, phi_here, T_here);
+    unstream_set<PS, SET_L>(K, t, pops, x, y, n, cell, phi_here, T_here);
 }
 
 // ---------------------------------------------------------------------------------------
