@@ -935,18 +935,33 @@ struct FieldOut {
     float sc[MAXF], lo[MAXF], hi[MAXF];
 };
 
-__global__ void pack_fields_kernel(FieldPtrs fp, int nfield, long long npix, int cin, bf16 *__restrict__ x)
+// A warp packs 32 pixels: each lane reads the fields of its pixel (coalesced) and
+// rounds them to one 16-byte chunk; the warp then writes the pixels' rows of cin / 8
+// chunks in order, 512 contiguous bytes per store, the field chunks passed by
+// shuffles.  Bound by the stores (2 cin bytes a pixel): one thread writing a pixel's
+// whole row took 75 us at 1024^2 (2.1 TB/s).
+__global__ void __launch_bounds__(256) pack_fields_kernel(FieldPtrs fp, int nfield, long long npix, int cin,
+                                                          bf16 *__restrict__ x)
 {
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
-         p += (long long)gridDim.x * blockDim.x) {
-        for (int c = 0; c < cin; c += 8) {
-            float v[8];
+    const int lane = threadIdx.x & 31, cv = cin / 8;
+    const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
+    for (long long g = blockIdx.x * (long long)(blockDim.x / 32) + threadIdx.x / 32; 32 * g < npix; g += nwarps) {
+        const long long p = 32 * g + lane;
+        float v[8];
 #pragma unroll
-            for (int e = 0; e < 8; e++) {
-                const int k = c + e;
-                v[e] = k < nfield ? (fp.f[k][p] - fp.off[k]) * fp.sc[k] : 0.0f;
-            }
-            *(uint4 *)(x + p * cin + c) = cnok::pack8(v);
+        for (int k = 0; k < 8; k++)
+            v[k] = (k < nfield && p < npix) ? (fp.f[k][p] - fp.off[k]) * fp.sc[k] : 0.0f;
+        const uint4 mine = cnok::pack8(v);
+        uint4 *row = (uint4 *)x + 32 * g * cv;
+        for (int j = 0; j < cv; j++) {
+            const int q = 32 * j + lane, pix = q / cv, chunk = q - pix * cv;
+            uint4 u;
+            u.x = __shfl_sync(0xffffffffu, mine.x, pix);
+            u.y = __shfl_sync(0xffffffffu, mine.y, pix);
+            u.z = __shfl_sync(0xffffffffu, mine.z, pix);
+            u.w = __shfl_sync(0xffffffffu, mine.w, pix);
+            if (32 * g + pix < npix)
+                row[q] = chunk == 0 ? u : make_uint4(0u, 0u, 0u, 0u);
         }
     }
 }
@@ -960,76 +975,198 @@ __global__ void pack_delta_kernel(FieldPtrs cur, FieldPtrs next, int nfield, lon
     }
 }
 
-__global__ void apply_update_kernel(FieldPtrs src, FieldOut dst, int nfield, long long npix,
-                                    const float *__restrict__ out, int out_cs, float phi_band)
+// All of a pixel's values are read before the first is written, so the reads of the
+// seven fields are in flight together (dst may equal src: the compiler may not move
+// reads over writes by itself; 31 us at 1024^2 before).
+__global__ void __launch_bounds__(256) apply_update_kernel(FieldPtrs src, FieldOut dst, int nfield, long long npix,
+                                                           const float *__restrict__ out, int out_cs, float phi_band)
 {
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
          p += (long long)gridDim.x * blockDim.x) {
-        for (int k = 0; k < nfield; k++) {
-            const float v = src.f[k][p];
-            const bool frozen = dst.sc[k] == 0.0f || (k == 0 && phi_band > 0.0f && fabsf(v) >= phi_band);
-            dst.f[k][p] = frozen ? v : fminf(fmaxf(v + dst.sc[k] * out[p * out_cs + k], dst.lo[k]), dst.hi[k]);
+        float v[MAXF], o[MAXF];
+#pragma unroll
+        for (int k = 0; k < MAXF; k++) {
+            v[k] = k < nfield ? src.f[k][p] : 0.0f;
+            o[k] = k < nfield && dst.sc[k] != 0.0f ? out[p * out_cs + k] : 0.0f;
         }
+#pragma unroll
+        for (int k = 0; k < MAXF; k++)
+            if (k < nfield) {
+                const bool frozen = dst.sc[k] == 0.0f || (k == 0 && phi_band > 0.0f && fabsf(v[k]) >= phi_band);
+                dst.f[k][p] = frozen ? v[k] : fminf(fmaxf(v[k] + dst.sc[k] * o[k], dst.lo[k]), dst.hi[k]);
+            }
     }
 }
 
-// per-row sums of phi, chi, f_s, 1 - phi^2, |grad phi|, the row's minimum and
-// maximum of T, and the sum of rho H (FP64), one block per row
+// Sums of phi, chi, f_s, 1 - phi^2, |grad phi|, the minimum and maximum of T, and
+// the sum of rho H.  FP64 is the scarce pipe of this GPU (2 lane operations per
+// cycle and SM), and evaluating and adding a cell's terms in FP64 took 114 us at
+// 1024^2.  Each term is formed as an unevaluated FP32 pair from error-free sums and
+// products (relative error of order 2^-44) and added with compensation, so that the
+// sums keep FP64 accuracy; only one conversion per warp and sum is left.  A cell with
+// a value beyond DIRECT (infinities and NaN among them), where the products could
+// overflow FP32, is evaluated and added in FP64.
 constexpr int NCHK = 8;
+constexpr float DIRECT = 1e12f;
 struct HCoef {
-    double cl, cs, cg, lat;
-    int on;
+    float cl, cs, cg, lat;
+    int on, wide;  // wide: a coefficient beyond DIRECT
 };
-__global__ void field_rows_kernel(const float *__restrict__ phi, const float *__restrict__ fs,
-                                  const float *__restrict__ T, HCoef hc, int nx, int ny, double *__restrict__ rows)
+struct ff {
+    float h, l;  // h + l, |l| small beside h
+};
+__device__ __forceinline__ ff ff_sum(float a, float b)  // exact
 {
-    __shared__ double red[NCHK][256];
-    const int y = blockIdx.x;
-    double s[NCHK] = {0, 0, 0, 0, 0, INFINITY, -INFINITY, 0};
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-        const long long c = (long long)y * nx + x;
-        const double f = phi[c];
-        const double fe = phi[(long long)y * nx + (x + 1) % nx], fw = phi[(long long)y * nx + (x + nx - 1) % nx];
-        double gy;
-        if (ny == 1)
-            gy = 0.0;
-        else if (y == 0)
-            gy = phi[c + nx] - f;
-        else if (y == ny - 1)
-            gy = f - phi[c - nx];
-        else
-            gy = 0.5 * (phi[c + nx] - phi[c - nx]);
-        const double gx = 0.5 * (fe - fw);
-        s[0] += f;
-        s[1] += fmin(fmax(0.5 * (1.0 + f), 0.0), 1.0);
-        s[2] += fs ? (double)fs[c] : 0.0;
-        s[3] += 1.0 - f * f;
-        s[4] += sqrt(gx * gx + gy * gy);
-        const double t = T ? (double)T[c] : 0.0;
-        s[5] = fmin(s[5], t);
-        s[6] = fmax(s[6], t);
-        if (hc.on) {
-            const double chi = fmin(fmax(0.5 * (1.0 + f), 0.0), 1.0);
-            const double sol = fmin(fmax((double)fs[c], 0.0), chi);
-            s[7] += t * (sol * hc.cs + (chi - sol) * hc.cl + (1.0 - chi) * hc.cg) + hc.lat * (chi - sol);
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ ff ff_add(ff a, ff b)
+{
+    const ff s = ff_sum(a.h, b.h);
+    return ff_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff ff_mul(ff a, ff b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    return {p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ ff ff_neg(ff a) { return {-a.h, -a.l}; }
+
+__device__ __forceinline__ void check_add(ff &a, ff x)
+{
+    const ff t = ff_sum(a.h, x.h);
+    a = {t.h, __fadd_rn(a.l, __fadd_rn(t.l, x.l))};
+}
+
+// A cell in FP64, added to the sums `wide`: f its phi, fe, fw, fn, fso the neighbours
+// (gradient scale gys in y).
+__device__ __noinline__ void check_wide(double (&wide)[6], double f, double fe, double fw, double fn, double fso, double gys,
+                                        double fs, double t, const HCoef &hc)
+{
+    const double gx = 0.5 * (fe - fw), gy = gys * (fn - fso);
+    const double chi = fmin(fmax(0.5 * (1.0 + f), 0.0), 1.0);
+    wide[0] += f;
+    wide[1] += chi;
+    wide[2] += fs;
+    wide[3] += 1.0 - f * f;
+    wide[4] += sqrt(gx * gx + gy * gy);
+    if (hc.on) {
+        const double sol = fmin(fmax(fs, 0.0), chi);
+        wide[5] += t * (sol * hc.cs + (chi - sol) * hc.cl + (1.0 - chi) * hc.cg) + (double)hc.lat * (chi - sol);
+    }
+}
+
+constexpr int CHK_THREADS = 256;
+__global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *__restrict__ phi, const float *__restrict__ fs,
+                                                                 const float *__restrict__ T, HCoef hc, int nx, int ny,
+                                                                 double *__restrict__ part)
+{
+    ff sum[6];       // phi, chi, f_s, 1 - phi^2, |grad phi|, rho H
+    double wide[6];  // the cells evaluated in FP64
+    float lo = INFINITY, hi = -INFINITY;  // T
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        sum[k] = {0.0f, 0.0f};
+        wide[k] = 0.0;
+    }
+    for (int y = blockIdx.x; y < ny; y += gridDim.x) {
+        const float *row = phi + (long long)y * nx;
+        // rows of the central difference in y, one-sided next to the walls
+        const float *rn = y + 1 < ny ? row + nx : row, *rs = y > 0 ? row - nx : row;
+        const float gys = y > 0 && y + 1 < ny ? 0.5f : 1.0f;
+        for (int x = threadIdx.x; x < nx; x += CHK_THREADS) {
+            const float f = row[x], fe = row[x + 1 < nx ? x + 1 : 0], fw = row[x > 0 ? x - 1 : nx - 1];
+            const float fn = rn[x], fso = rs[x];
+            const float sol = fs ? fs[(long long)y * nx + x] : 0.0f, t = T ? T[(long long)y * nx + x] : 0.0f;
+            lo = fminf(lo, t);
+            hi = fmaxf(hi, t);
+            const float mag = fmaxf(fmaxf(fabsf(f), fabsf(sol)), fabsf(t));
+            const float nb = fmaxf(fmaxf(fabsf(fe), fabsf(fw)), fmaxf(fabsf(fn), fabsf(fso)));
+            const float all = fabsf(f) + fabsf(sol) + fabsf(t) + fabsf(fe) + fabsf(fw) + fabsf(fn) + fabsf(fso);  // NaN kept
+            if (hc.wide || !(fmaxf(mag, nb) < DIRECT) || !(all < INFINITY)) {
+                check_wide(wide, f, fe, fw, fn, fso, gys, sol, t, hc);
+                continue;
+            }
+            check_add(sum[0], {f, 0.0f});
+            // chi = clamp((1 + phi) / 2)
+            ff chi = ff_sum(1.0f, f);
+            chi = {0.5f * chi.h, 0.5f * chi.l};
+            if (!(f > -1.0f)) chi = {0.0f, 0.0f};
+            if (!(f < 1.0f)) chi = {1.0f, 0.0f};
+            check_add(sum[1], chi);
+            check_add(sum[2], {sol, 0.0f});
+            const ff ff0 = {f, 0.0f};
+            check_add(sum[3], ff_add({1.0f, 0.0f}, ff_neg(ff_mul(ff0, ff0))));
+            // |grad phi| = sqrt(gx^2 + gy^2): FP32 root and one Newton correction
+            ff gx = ff_sum(fe, -fw), gy = ff_sum(fn, -fso);
+            gx = {0.5f * gx.h, 0.5f * gx.l};
+            gy = {gys * gy.h, gys * gy.l};
+            const ff q = ff_add(ff_mul(gx, gx), ff_mul(gy, gy));
+            const float r = sqrtf(q.h);
+            if (r > 0.0f) {
+                const float res = __fadd_rn(__fmaf_rn(-r, r, q.h), q.l);
+                check_add(sum[4], {r, __fdiv_rn(res, 2.0f * r)});
+            }
+            if (hc.on) {
+                // sol = clamp(f_s, 0, chi); rho H = T (sol c_s + d c_l + (1 - chi) c_g) + lat d, d = chi - sol
+                ff so = {fmaxf(sol, 0.0f), 0.0f};
+                if (so.h > chi.h || (so.h == chi.h && chi.l < 0.0f)) so = chi;
+                const ff d = ff_add(chi, ff_neg(so)), gas = ff_add({1.0f, 0.0f}, ff_neg(chi));
+                const ff cap = ff_add(ff_add(ff_mul(so, {hc.cs, 0.0f}), ff_mul(d, {hc.cl, 0.0f})), ff_mul(gas, {hc.cg, 0.0f}));
+                check_add(sum[5], ff_add(ff_mul({t, 0.0f}, cap), ff_mul(d, {hc.lat, 0.0f})));
+            }
         }
     }
-    for (int k = 0; k < NCHK; k++)
-        red[k][threadIdx.x] = s[k];
+    // the warp's sums in a fixed order, still as pairs, then the block's in FP64
+    __shared__ double red[CHK_THREADS / 32][NCHK];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    bool any_wide = false;
+#pragma unroll
+    for (int k = 0; k < 6; k++) any_wide = any_wide || wide[k] != 0.0;  // true for NaN too
+    any_wide = __any_sync(0xffffffffu, any_wide);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        ff v = sum[k];
+        for (int o = 16; o > 0; o >>= 1) {
+            const ff u = {__shfl_down_sync(0xffffffffu, v.h, o), __shfl_down_sync(0xffffffffu, v.l, o)};
+            check_add(v, u);
+        }
+        double s = (double)v.h + (double)v.l;
+        if (any_wide) {
+            double wd = wide[k];
+            for (int o = 16; o > 0; o >>= 1) wd += __shfl_down_sync(0xffffffffu, wd, o);
+            s += wd;
+        }
+        if (lane == 0) red[w][k < 5 ? k : 7] = s;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_down_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_down_sync(0xffffffffu, hi, o));
+    }
+    if (lane == 0) {
+        red[w][5] = lo;
+        red[w][6] = hi;
+    }
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            for (int k = 0; k < 5; k++)
-                red[k][threadIdx.x] += red[k][threadIdx.x + st];
-            red[5][threadIdx.x] = fmin(red[5][threadIdx.x], red[5][threadIdx.x + st]);
-            red[6][threadIdx.x] = fmax(red[6][threadIdx.x], red[6][threadIdx.x + st]);
-            red[7][threadIdx.x] += red[7][threadIdx.x + st];
-        }
-        __syncthreads();
+    if (threadIdx.x < NCHK) {
+        const int k = threadIdx.x;
+        double s = red[0][k];
+        for (int j = 1; j < CHK_THREADS / 32; j++)
+            s = k == 5 ? fmin(s, red[j][k]) : (k == 6 ? fmax(s, red[j][k]) : s + red[j][k]);
+        part[(long long)blockIdx.x * NCHK + k] = s;
     }
-    if (threadIdx.x == 0)
-        for (int k = 0; k < NCHK; k++)
-            rows[NCHK * y + k] = red[k][0];
+}
+
+// The blocks' sums in a fixed order: thread (k, j) takes blocks j, j + 32, ...
+__global__ void __launch_bounds__(32 * NCHK) field_total_kernel(const double *__restrict__ part, int blocks,
+                                                                double *__restrict__ out)
+{
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto join = [&](double a, double b) { return k == 5 ? fmin(a, b) : (k == 6 ? fmax(a, b) : a + b); };
+    double s = k == 5 ? INFINITY : (k == 6 ? -INFINITY : 0.0);
+    for (int b = lane; b < blocks; b += 32) s = join(s, part[(long long)b * NCHK + k]);
+    for (int o = 16; o > 0; o >>= 1) s = join(s, __shfl_down_sync(0xffffffffu, s, o));
+    if (lane == 0) out[k] = s;
 }
 }  // namespace
 
@@ -1108,29 +1245,26 @@ extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const 
 {
     if (!phi || !out || nx < 1 || ny < 1)
         return fail(CNO_ERR_INVALID_ARG, "bad check arguments");
-    double *rows = nullptr;
-    CK(cudaMallocAsync(&rows, (size_t)ny * NCHK * sizeof(double), (cudaStream_t)stream));
-    HCoef hc = {0, 0, 0, 0, 0};
-    if (hcoef && fs && T)
-        hc = {hcoef[0], hcoef[1], hcoef[2], hcoef[3], 1};
-    field_rows_kernel<<<ny, 256, 0, (cudaStream_t)stream>>>(phi, fs, T, hc, nx, ny, rows);
-    CK(cudaGetLastError());
-    std::vector<double> h((size_t)ny * NCHK);
-    CK(cudaMemcpyAsync(h.data(), rows, h.size() * sizeof(double), cudaMemcpyDeviceToHost, (cudaStream_t)stream));
-    CK(cudaFreeAsync(rows, (cudaStream_t)stream));
-    CK(cudaStreamSynchronize((cudaStream_t)stream));
-    for (int k = 0; k < 5; k++)
-        out[k] = 0.0;
-    out[5] = INFINITY;
-    out[6] = -INFINITY;
-    out[7] = 0.0;
-    for (int y = 0; y < ny; y++) {
-        for (int k = 0; k < 5; k++)
-            out[k] += h[(size_t)NCHK * y + k];
-        out[5] = std::min(out[5], h[(size_t)NCHK * y + 5]);
-        out[6] = std::max(out[6], h[(size_t)NCHK * y + 6]);
-        out[7] += h[(size_t)NCHK * y + 7];
+    cudaStream_t st = (cudaStream_t)stream;
+    const int blocks = std::min(ny, 4 * num_sms());
+    double *part = nullptr;
+    CK(cudaMallocAsync(&part, (size_t)(blocks + 1) * NCHK * sizeof(double), st));
+    HCoef hc = {0, 0, 0, 0, 0, 0};
+    if (hcoef && fs && T) {
+        hc = {hcoef[0], hcoef[1], hcoef[2], hcoef[3], 1, 0};
+        for (int k = 0; k < 4; k++)
+            if (!(std::fabs(hcoef[k]) < DIRECT))
+                hc.wide = 1;
     }
+    field_sums_kernel<<<blocks, CHK_THREADS, 0, st>>>(phi, fs, T, hc, nx, ny, part + NCHK);
+    field_total_kernel<<<1, 32 * NCHK, 0, st>>>(part + NCHK, blocks, part);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out, part, NCHK * sizeof(double), cudaMemcpyDeviceToHost, st);
+    const cudaError_t fe = cudaFreeAsync(part, st);
+    CK(e);
+    CK(fe);
+    CK(cudaStreamSynchronize(st));
     if (!T)
         out[5] = out[6] = 0.0;
     return CNO_OK;

@@ -86,3 +86,68 @@ def test_device_read_out_matches_host(nx, ny):
     for i in range(3):
         rest[1 + i * (nx * ny + 1):1 + i * (nx * ny + 1) + nx * ny] = False
     assert bool((buf[rest] == 7.5).all())
+
+
+def _checks(phi, fs, T, hc):
+    """The acceptance checks in FP64 numpy, as long sums."""
+    p, f, t = (a.astype(np.longdouble) for a in (phi, fs, T))
+    gx = 0.5 * (np.roll(p, -1, 1) - np.roll(p, 1, 1))
+    gy = np.zeros_like(p)
+    if len(p) > 1:
+        gy[1:-1], gy[0], gy[-1] = 0.5 * (p[2:] - p[:-2]), p[1] - p[0], p[-1] - p[-2]
+    chi = np.clip(0.5 * (1 + p), 0, 1)
+    sol = np.minimum(np.maximum(f, 0), chi)
+    H = t * (sol * hc[1] + (chi - sol) * hc[0] + (1 - chi) * hc[2]) + hc[3] * (chi - sol)
+    return [v.sum() for v in (p, chi, f, 1 - p * p, np.sqrt(gx * gx + gy * gy))] + [t.min(), t.max(), H.sum()]
+
+
+# one row, two rows, more columns than threads, more rows than blocks; values up to and beyond the FP32 form's range
+@pytest.mark.parametrize("nx,ny", [(1, 1), (5, 2), (33, 3), (300, 7), (17, 1300), (512, 96)])
+@pytest.mark.parametrize("scale", [1.0, 1e-12, 1e14])
+def test_field_checks_keep_fp64_accuracy(nx, ny, scale):
+    from paper_2511_09422_gb300 import cno
+    rng = np.random.default_rng(nx + ny)
+    phi = np.tanh(rng.standard_normal((ny, nx)) * 3).astype(np.float32)
+    phi[rng.random((ny, nx)) < 0.05] *= np.float32(1.1 * scale)
+    fs = (rng.uniform(-0.1, 1.1, (ny, nx))).astype(np.float32)
+    T = (scale * rng.standard_normal((ny, nx))).astype(np.float32)
+    hc = tuple(float(np.float32(v)) for v in (1.0, 0.9, 0.37, 11.3))
+    got = cno.field_checks(*(torch.as_tensor(a).cuda() for a in (phi, fs, T)), hc)
+    want = _checks(phi, fs, T, hc)
+    mags = _checks(np.abs(phi), np.abs(fs), np.abs(T), hc)
+    for k in range(8):  # FP64 sums of N terms: N 2^-53 of the terms' magnitudes; 1 - phi^2 of 1 + phi^2
+        mag = abs(mags[k]) + (2 * nx * ny + 2 * float((phi.astype(np.float64) ** 2).sum()) if k == 3 else 0)
+        mag += (2 * nx * ny * 12 if k == 7 else 0)
+        assert abs(got[k] - want[k]) <= 1e-12 * float(mag) + 1e-300, (k, got[k], want[k])
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_field_checks_with_non_finite_values(bad):
+    from paper_2511_09422_gb300 import cno
+    rng = np.random.default_rng(1)
+    phi, fs, T = (rng.uniform(0.1, 0.9, (40, 50)).astype(np.float32) for _ in range(3))
+    hc = (1.0, 0.9, 0.4, 11.0)
+    clean = cno.field_checks(*(torch.as_tensor(a).cuda() for a in (phi, fs, T)), hc)
+    T[20, 30] = bad
+    got = cno.field_checks(*(torch.as_tensor(a).cuda() for a in (phi, fs, T)), hc)
+    assert got[:5] == pytest.approx(clean[:5], rel=1e-14)
+    assert np.isnan(got[7]) if np.isnan(bad) else got[7] == bad
+    phi[3, 3] = bad
+    got = cno.field_checks(*(torch.as_tensor(a).cuda() for a in (phi, fs, T)), hc)
+    assert not np.isfinite(got[0]) and not np.isfinite(got[3]) and not np.isfinite(got[4]) and np.isfinite(got[1])
+
+
+@pytest.mark.parametrize("nx,ny,cin,nfield", [(1, 1, 8, 1), (31, 3, 64, 7), (32, 1, 64, 8), (100, 33, 24, 5), (64, 64, 256, 7)])
+def test_pack_fields_rounds_and_pads(nx, ny, cin, nfield):
+    from paper_2511_09422_gb300 import cno
+    gen = torch.Generator(device="cuda").manual_seed(nx)
+    f = [torch.randn((ny, nx), device="cuda", generator=gen) for _ in range(nfield)]
+    off, sc = np.linspace(-1, 1, nfield).astype(np.float32), np.linspace(0.5, 3, nfield).astype(np.float32)
+    buf = torch.full((ny * nx * cin + 8,), 3.0, dtype=torch.bfloat16, device="cuda")
+    x = buf[:ny * nx * cin].view(1, ny, nx, cin)
+    cno.pack_fields(f, off, sc, cin=cin, out=x)
+    want = torch.zeros((1, ny, nx, cin), dtype=torch.bfloat16, device="cuda")
+    for k in range(nfield):
+        want[0, ..., k] = ((f[k] - float(off[k])) * float(sc[k])).to(torch.bfloat16)
+    assert torch.equal(x, want)
+    assert bool((buf[ny * nx * cin:] == 3.0).all())
