@@ -153,6 +153,24 @@ static int num_sms()
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
+// Launch with programmatic dependent launch (the kernel calls grid_begin): its
+// blocks start while the last blocks of the kernel in front of it finish.
+template <class... P, class... A>
+static cudaError_t launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 static bool chan_ok(int c) { return c >= 64 && c % 64 == 0 && c <= 4096; }
 
 static cno_status check_image(int n, int h, int w)
@@ -188,8 +206,7 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
     // persistent: at most the CTAs that fit on the SMs at once
     const int ctas = std::min(tiles, S::CTAS_PER_SM * num_sms());
     dim3 grid(ctas, a.cout / BN);
-    cnok::conv_fprop_kernel<BN><<<grid, 192, S::SMEM, st>>>(mx, mw, a);
-    CK(cudaGetLastError());
+    CK(launch(cnok::conv_fprop_kernel<BN>, grid, 192, S::SMEM, st, mx, mw, a));
     return CNO_OK;
 }
 
@@ -197,7 +214,8 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
 // (epi = SLOPE / PLAIN) convolutions: out[p][o] = sum_{t,i} in[p + s_t][i] wmat[o][t][i].
 static cno_status conv_launch(const void *in, int n, int h, int w, int cin, const void *wmat, int cout, int epi,
                               const float *bias, const void *slope_src, void *out, int out_f32, int out_cs,
-                              int n_store, unsigned *status, cudaStream_t st)
+                              int n_store, unsigned *status, cudaStream_t st, float *out2 = nullptr, int out2_cs = 0,
+                              int n2 = 0)
 {
     CS(check_image(n, h, w));
     if (!chan_ok(cin) || !chan_ok(cout))
@@ -234,6 +252,9 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
     a.out_cs = out_cs;
     a.n_store = n_store;
     a.out_f32 = out_f32;
+    a.out2 = out2;
+    a.out2_cs = out2_cs;
+    a.n2 = n2;
     a.status = status;
     const long long tiles = (long long)n * a.tiles_w * a.tiles_h;
     if (tiles > 0x7fffffffLL)
@@ -256,8 +277,7 @@ static cno_status launch_wgrad_bn(const CUtensorMap &mdz, const CUtensorMap &mx,
         attr = true;
     }
     dim3 grid(9 * a.mtiles * a.ntiles, a.splits);
-    cnok::conv_wgrad_kernel<BN><<<grid, 192, S::SMEM, st>>>(mdz, mx, a);
-    CK(cudaGetLastError());
+    CK(launch(cnok::conv_wgrad_kernel<BN>, grid, 192, S::SMEM, st, mdz, mx, a));
     return CNO_OK;
 }
 
@@ -338,18 +358,15 @@ static cno_status wgrad_launch(const void *dz, const void *x, int n, int h, int 
     default: CS(launch_wgrad_bn<64>(mdz, mx, a, st)); break;
     }
     const long long count = (long long)cout * 9 * cin;
-    cnok::sum_partials_kernel<<<grid_for(count, 256), 256, 0, st>>>(partial, a.splits, count, dw);
-    CK(cudaGetLastError());
+    CK(launch(cnok::sum_partials_kernel, grid_for(count, 256), 256, 0, st, partial, a.splits, count, dw));
     if (db) {
         // bias gradient: per-block channel sums, then the blocks in order (the
         // same stream orders this after the weight sum above)
         const long long npix = (long long)n * h * w;
         const int blocks = bias_blocks(n, h, w);
         const long long ppb = (npix + blocks - 1) / blocks;
-        cnok::channel_sum_kernel<<<blocks, 256, 0, st>>>((const bf16 *)dz, npix, cout, ppb, partial);
-        CK(cudaGetLastError());
-        cnok::sum_partials_kernel<<<grid_for(cout, 256), 256, 0, st>>>(partial, blocks, cout, db);
-        CK(cudaGetLastError());
+        CK(launch(cnok::channel_sum_kernel, blocks, 256, 0, st, (const bf16 *)dz, npix, cout, ppb, partial));
+        CK(launch(cnok::channel_total_kernel, (cout + 31) / 32, 1024, 0, st, partial, blocks, cout, db));
     }
     return CNO_OK;
 }
@@ -436,9 +453,8 @@ extern "C" cno_status cno_weights_to_bf16(const float *w, int cout, int cin, voi
     if (!w || !wf || !wd || cout < 1 || cin < 1)
         return fail(CNO_ERR_INVALID_ARG, "bad weight conversion arguments");
     const long long total = (long long)cout * 9 * cin;
-    cnok::weights_to_bf16_kernel<<<grid_for(total, 256), 256, 0, (cudaStream_t)stream>>>(w, cout, cin, (bf16 *)wf,
-                                                                                         (bf16 *)wd);
-    CK(cudaGetLastError());
+    CK(launch(cnok::weights_to_bf16_kernel, grid_for(total, 256), 256, 0, (cudaStream_t)stream, w, cout, cin, (bf16 *)wf,
+              (bf16 *)wd));
     return CNO_OK;
 }
 
@@ -729,13 +745,15 @@ extern "C" cno_status cno_get_grads(cno_net *net, float *host)
     return CNO_OK;
 }
 
-static cno_status fwd_conv(cno_net *net, int k, const bf16 *in, int lv, bf16 *out_bf)
+// out2 (the head, k = 11): the caller's output, out2_cs channels per pixel, beside the network's own.
+static cno_status fwd_conv(cno_net *net, int k, const bf16 *in, int lv, bf16 *out_bf, float *out2 = nullptr,
+                           int out2_cs = 0)
 {
     const Layer &L = net->layers[k];
     const int h = net->ah >> lv, w = net->aw >> lv;
     if (k == 11)
         return conv_launch(in, net->an, h, w, L.cin, net->wf[k], L.cout, cnok::EPI_BIAS, net->p + L.b_off, nullptr,
-                           net->out, 1, 8, 8, net->status, net->st);
+                           net->out, 1, 8, 8, net->status, net->st, out2, out2_cs, net->nf);
     return conv_launch(in, net->an, h, w, L.cin, net->wf[k], L.cout, cnok::EPI_BIAS_LRELU, net->p + L.b_off, nullptr,
                        out_bf, 0, L.cout, L.cout, net->status, net->st);
 }
@@ -744,8 +762,7 @@ static cno_status pool(cno_net *net, const bf16 *x, int lv_out, int c, bf16 *y)
 {
     const int ho = net->ah >> lv_out, wo = net->aw >> lv_out;
     const long long total = (long long)net->an * ho * wo * (c / 8);
-    cnok::pool2_kernel<<<grid_for(total, 256), 256, 0, net->st>>>(x, net->an, ho, wo, c, y);
-    CK(cudaGetLastError());
+    CK(launch(cnok::pool2_kernel, grid_for(total, 256), 256, 0, net->st, x, net->an, ho, wo, c, y));
     return CNO_OK;
 }
 
@@ -753,12 +770,11 @@ static cno_status up_add(cno_net *net, const bf16 *x, const bf16 *skip, int lv_o
 {
     const int h = net->ah >> lv_out, w = net->aw >> lv_out;
     const long long total = (long long)net->an * h * w * (c / 8);
-    cnok::up_add_kernel<<<grid_for(total, 256), 256, 0, net->st>>>(x, skip, net->an, h, w, c, u);
-    CK(cudaGetLastError());
+    CK(launch(cnok::up_add_kernel, grid_for(total, 256), 256, 0, net->st, x, skip, net->an, h, w, c, u));
     return CNO_OK;
 }
 
-static cno_status forward_all(cno_net *net, const bf16 *x)
+static cno_status forward_all(cno_net *net, const bf16 *x, float *out = nullptr, int out_cs = 0)
 {
     auto &A = net->act;
     const int c0 = net->widths[0], c1 = net->widths[1], c2 = net->widths[2];
@@ -780,7 +796,7 @@ static cno_status forward_all(cno_net *net, const bf16 *x)
     CS(fwd_conv(net, 9, A[A_U1], 1, A[A_D1]));
     CS(up_add(net, A[A_D1], A[A_E0], 0, c0, A[A_U0]));
     CS(fwd_conv(net, 10, A[A_U0], 0, A[A_D0]));
-    CS(fwd_conv(net, 11, A[A_D0], 0, nullptr));
+    CS(fwd_conv(net, 11, A[A_D0], 0, nullptr, out, out_cs));
     return CNO_OK;
 }
 
@@ -791,8 +807,19 @@ extern "C" cno_status cno_forward(cno_net *net, const void *x, int n, int h, int
     if (out && out_cs < net->nf)
         return fail(CNO_ERR_INVALID_ARG, "out_cs must be at least nf");
     CS(ensure_buffers(net, n, h, w, false));
-    CS(forward_all(net, (const bf16 *)x));
-    if (out) {
+    // The head writes the caller's channels itself where they lie in this device's memory: a
+    // copy of the rows of nf floats took 94 us at 1024^2.
+    cudaPointerAttributes pa;
+    int dev = -1;
+    bool direct = false;
+    if (out && !((uintptr_t)out & 3) && cudaGetDevice(&dev) == cudaSuccess) {
+        if (cudaPointerGetAttributes(&pa, out) == cudaSuccess)
+            direct = pa.type == cudaMemoryTypeDevice && pa.device == dev;
+        else
+            cudaGetLastError();
+    }
+    CS(forward_all(net, (const bf16 *)x, direct ? out : nullptr, out_cs));
+    if (out && !direct) {
         CK(cudaMemcpy2DAsync(out, (size_t)out_cs * sizeof(float), net->out, 8 * sizeof(float),
                              net->nf * sizeof(float), (size_t)n * h * w, cudaMemcpyDeviceToDevice, net->st));
     }
@@ -826,8 +853,7 @@ static cno_status up_bwd(cno_net *net, const bf16 *du, const bf16 *y, int lv_out
 {
     const int ho = net->ah >> lv_out, wo = net->aw >> lv_out;
     const long long total = (long long)net->an * ho * wo * (c / 8);
-    cnok::up_bwd_kernel<<<grid_for(total, 256), 256, 0, net->st>>>(du, y, net->an, ho, wo, c, dz);
-    CK(cudaGetLastError());
+    CK(launch(cnok::up_bwd_kernel, grid_for(total, 256), 256, 0, net->st, du, y, net->an, ho, wo, c, dz));
     return CNO_OK;
 }
 
@@ -835,8 +861,7 @@ static cno_status pool_bwd(cno_net *net, const bf16 *du, const bf16 *dp, const b
 {
     const int h = net->ah >> lv, w = net->aw >> lv;
     const long long total = (long long)net->an * h * w * (c / 8);
-    cnok::pool_bwd_kernel<<<grid_for(total, 256), 256, 0, net->st>>>(du, dp, e, net->an, h, w, c, dz);
-    CK(cudaGetLastError());
+    CK(launch(cnok::pool_bwd_kernel, grid_for(total, 256), 256, 0, net->st, du, dp, e, net->an, h, w, c, dz));
     return CNO_OK;
 }
 
@@ -894,19 +919,15 @@ extern "C" cno_status cno_train_step(cno_net *net, const void *x, const float *t
     CS(forward_all(net, (const bf16 *)x));
     const long long npix = (long long)n * h * w;
     const unsigned blocks = std::min<unsigned>(4096u, grid_for(npix, 256));
-    cnok::mse_kernel<<<blocks, 256, 0, net->st>>>(net->out, 8, target, net->nf, npix, net->cout,
-                                                  1.0 / ((double)npix * net->nf), net->dout, net->loss_partial);
-    CK(cudaGetLastError());
+    CK(launch(cnok::mse_kernel, blocks, 256, 0, net->st, net->out, target, net->nf, npix, net->cout,
+              1.0 / ((double)npix * net->nf), net->dout, net->loss_partial));
     CS(backward_all(net, (const bf16 *)x));
     if (update) {
         net->step++;
         const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
         const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
-        cnok::adam_kernel<<<grid_for(net->nparams, 256), 256, 0, net->st>>>(net->p, net->g, net->m, net->v,
-                                                                            net->nparams, lr, 0.9f, 0.999f,
-                                                                            (float)(1.0 - 0.9), (float)(1.0 - 0.999),
-                                                                            1e-8f, c1, c2);
-        CK(cudaGetLastError());
+        CK(launch(cnok::adam_kernel, grid_for(net->nparams, 256), 256, 0, net->st, net->p, net->g, net->m, net->v,
+                  net->nparams, lr, 0.9f, 0.999f, (float)(1.0 - 0.9), (float)(1.0 - 0.999), 1e-8f, c1, c2));
         CS(refresh_bf16(net));
     }
     if (loss) {

@@ -31,6 +31,17 @@ constexpr unsigned ST_TIMEOUT_PRODUCER = 1u, ST_TIMEOUT_MMA = 2u, ST_TIMEOUT_EPI
 // --------------------------------------------------------------------------
 // PTX wrappers
 // --------------------------------------------------------------------------
+// Programmatic dependent launch: the blocks of a kernel may be resident before the
+// kernel in front of it has ended.  grid_begin waits for that kernel's end (its
+// writes are then visible) and only then lets the kernel behind this one start its
+// blocks, so at most two are ever in flight.  Every kernel launched that way calls
+// it before its first access to global memory.
+__device__ __forceinline__ void grid_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -235,6 +246,8 @@ struct ConvArgs {
     const bf16 *slope_src;      // EPI_SLOPE: y whose lrelu slope multiplies the result (NHWC, cout channels)
     void *out;                  // NHWC, out_cs channels per pixel
     int out_cs, n_store, out_f32;
+    float *out2;                // FP32 outputs only: the first n2 <= min(8, n_store) channels again, out2_cs per pixel
+    int out2_cs, n2;
     unsigned *status;
 };
 
@@ -259,8 +272,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// (At BN = 64 the bound keeps the kernel at 96 registers: with 104 a scheduler's
+// register file holds four warps instead of five, so two CTAs fit instead of three
+// and the 64-channel layers take 25 % longer.)
 template <int BN>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
     conv_fprop_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                       const ConvArgs a)
 {
@@ -275,6 +291,7 @@ __global__ void __launch_bounds__(192, 1)
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
     float *sbias = (float *)(smem + S::STAGES * S::STAGE + S::BAR_BYTES);
 
+    grid_begin();
     if (*(volatile unsigned *)a.status != 0u)
         return;  // an earlier launch failed: leave the output untouched
 
@@ -418,8 +435,18 @@ __global__ void __launch_bounds__(192, 1)
                 }
                 const int nst = min(32, a.n_store - oc);
                 if (a.out_f32) {
+                    if (a.out2 && oc == 0) {
+                        float *o2 = a.out2 + pix * a.out2_cs;
+#pragma unroll
+                        for (int i = 0; i < 8; i++)
+                            if (i < a.n2)
+                                o2[i] = v[i];
+                    }
                     float *o = (float *)a.out + pix * a.out_cs + oc;
-                    if (nst == 32 && (a.out_cs & 3) == 0) {
+                    if (nst == 8 && (a.out_cs & 3) == 0) {
+                        ((float4 *)o)[0] = make_float4(v[0], v[1], v[2], v[3]);
+                        ((float4 *)o)[1] = make_float4(v[4], v[5], v[6], v[7]);
+                    } else if (nst == 32 && (a.out_cs & 3) == 0) {
 #pragma unroll
                         for (int j = 0; j < 8; j++)
                             ((float4 *)o)[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
@@ -506,6 +533,7 @@ __global__ void __launch_bounds__(192, 1)
     uint32_t *tmem_holder = (uint32_t *)(done + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
 
+    grid_begin();
     if (*(volatile unsigned *)a.status != 0u)
         return;
 
@@ -653,14 +681,25 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8])
     return u;
 }
 
-// dW[i] = sum over splits s (in order) of partial[s][i]
-__global__ void sum_partials_kernel(const float *__restrict__ partial, int splits, long long count,
-                                    float *__restrict__ out)
+// dW[i] = sum over splits s (in order) of partial[s][i]; eight reads in flight
+__global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restrict__ partial, int splits,
+                                                           long long count, float *__restrict__ out)
 {
+    grid_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x) {
         float s = 0.0f;
-        for (int k = 0; k < splits; k++)
+        int k = 0;
+        for (; k + 8 <= splits; k += 8) {
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                v[e] = partial[(k + e) * count + i];
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                s += v[e];
+        }
+        for (; k < splits; k++)
             s += partial[k * count + i];
         out[i] = s;
     }
@@ -670,10 +709,12 @@ __global__ void sum_partials_kernel(const float *__restrict__ partial, int split
 // range [b * ppb, (b + 1) * ppb) per channel into partial[b][c].  Thread t reads
 // 8 channels (16 bytes) of pixel p0 + t / (c / 8) + k * (256 / (c / 8)), so a
 // warp's loads are contiguous; the threads of one channel group are then added
-// in shared memory in a fixed order.
+// in shared memory in a fixed order.  Bound by the read of dz: each thread keeps
+// eight loads in flight (with one, 50 us for 134 MB, 2.7 TB/s).
 __global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *__restrict__ dz, long long npix, int c,
                                                           long long ppb, float *__restrict__ partial)
 {
+    grid_begin();
     __shared__ float red[256][9];
     const int groups = c / 8;                 // 16-byte channel groups (c <= 2048)
     const int lanes_per_pix = groups;
@@ -682,14 +723,27 @@ __global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *__restrict
     const long long p0 = (long long)blockIdx.x * ppb;
     const long long p1 = min(npix, p0 + ppb);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (r < pix_step) {
-        for (long long p = p0 + r; p < p1; p += pix_step) {
-            float f[8];
-            unpack8(*(const uint4 *)(dz + p * c + 8 * g), f);
+    auto add = [&](uint4 u) {
+        float f[8];
+        unpack8(u, f);
 #pragma unroll
-            for (int e = 0; e < 8; e++)
-                acc[e] += f[e];
+        for (int e = 0; e < 8; e++)
+            acc[e] += f[e];
+    };
+    if (r < pix_step) {
+        const uint4 *src = (const uint4 *)(dz + 8 * g);
+        long long p = p0 + r;
+        for (; p + 7 * pix_step < p1; p += 8 * pix_step) {
+            uint4 u[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                u[j] = src[(p + j * pix_step) * groups];
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                add(u[j]);
         }
+        for (; p < p1; p += pix_step)
+            add(src[p * groups]);
     }
 #pragma unroll
     for (int e = 0; e < 8; e++)
@@ -704,12 +758,35 @@ __global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *__restrict
     }
 }
 
+// Bias gradient, second pass: db[ch] = sum of partial[b][ch] over the blocks, one
+// block of 32 channels x 32 block groups, added in a fixed order.
+__global__ void __launch_bounds__(1024) channel_total_kernel(const float *__restrict__ partial, int blocks, int c,
+                                                             float *__restrict__ db)
+{
+    grid_begin();
+    __shared__ float red[32][33];
+    const int lane = threadIdx.x & 31, j = threadIdx.x >> 5, ch = blockIdx.x * 32 + lane;
+    float s = 0.0f;
+    if (ch < c)
+        for (int b = j; b < blocks; b += 32)
+            s += partial[(long long)b * c + ch];
+    red[j][lane] = s;
+    __syncthreads();
+    // warp j adds the 32 group sums of channel j by a tree
+    float t = red[lane][j];
+    for (int o = 16; o > 0; o >>= 1)
+        t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0 && blockIdx.x * 32 + j < c)
+        db[blockIdx.x * 32 + j] = t;
+}
+
 // --------------------------------------------------------------------------
 // Elementwise kernels on NHWC bf16 tensors, 8 channels (16 bytes) per thread.
 // --------------------------------------------------------------------------
 // y[n][h][w] = mean of x[n][2h..2h+1][2w..2w+1]; x is n x 2ho x 2wo
 __global__ void pool2_kernel(const bf16 *__restrict__ x, int n, int ho, int wo, int c, bf16 *__restrict__ y)
 {
+    grid_begin();
     const int cv = c / 8;
     const long long total = (long long)n * ho * wo * cv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -744,6 +821,7 @@ __global__ void pool2_kernel(const bf16 *__restrict__ x, int n, int ho, int wo, 
 __global__ void up_add_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ skip, int n, int h, int w, int c,
                               bf16 *__restrict__ u)
 {
+    grid_begin();
     const int cv = c / 8;
     const long long total = (long long)n * h * w * cv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -770,6 +848,7 @@ __global__ void up_add_kernel(const bf16 *__restrict__ x, const bf16 *__restrict
 __global__ void up_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restrict__ y, int n, int ho, int wo, int c,
                               bf16 *__restrict__ dz)
 {
+    grid_begin();
     const int cv = c / 8;
     const long long total = (long long)n * ho * wo * cv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -808,6 +887,7 @@ __global__ void up_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restric
 __global__ void pool_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restrict__ dp, const bf16 *__restrict__ e,
                                 int n, int h, int w, int c, bf16 *__restrict__ dz)
 {
+    grid_begin();
     const int cv = c / 8;
     const long long total = (long long)n * h * w * cv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -830,43 +910,75 @@ __global__ void pool_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restr
     }
 }
 
-// Mean squared error over the first nf channels of out (FP32, out_cs per
-// pixel) against target (FP32, nf per pixel).  dout (bf16, c per pixel) gets
-// 2 (out - target) / count on those channels and 0 elsewhere; each block adds
-// its squared errors in FP64 into partial[block].
-__global__ void mse_kernel(const float *__restrict__ out, int out_cs, const float *__restrict__ target, int nf,
-                           long long npix, int c, double inv_count, bf16 *__restrict__ dout,
-                           double *__restrict__ partial)
+// Mean squared error over the first nf <= 8 channels of out (FP32, 8 per pixel)
+// against target (FP32, nf per pixel).  dout (bf16, c per pixel) gets 2 (out -
+// target) / count on those channels and 0 elsewhere; each block adds its squared
+// errors into partial[block] (FP64).  A warp takes 32 pixels: each lane forms the
+// gradient of its pixel, and the warp writes the pixels' rows in order, 512
+// contiguous bytes per store.  The squares are summed as exact FP32 pairs with
+// compensation.  Bound by the write of dout; in FP64, one row per thread, this
+// took 259 us for 16 x 256^2 (134 MB).
+__global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ out, const float *__restrict__ target,
+                                                  int nf, long long npix, int c, double inv_count,
+                                                  bf16 *__restrict__ dout, double *__restrict__ partial)
 {
-    __shared__ double red[256];
-    double acc = 0.0;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
-         p += (long long)gridDim.x * blockDim.x) {
-        for (int ch = 0; ch < c; ch += 8) {
-            float g[8];
+    grid_begin();
+    __shared__ double red[8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cv = c / 8;
+    const float scale = (float)(2.0 * inv_count);
+    float hi = 0.0f, lo = 0.0f;  // sum of squares
+    double wide = 0.0;           // of differences beyond 1e12, NaN and infinities
+    auto add = [&](float x, float e) {  // hi + lo += x + e, the rounding error kept
+        const float s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb))));
+        hi = s;
+    };
+    for (long long g = blockIdx.x * 8LL + w; 32 * g < npix; g += gridDim.x * 8LL) {
+        const long long p = 32 * g + lane;
+        float d[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (p < npix) {
+            const float4 a = ((const float4 *)out)[2 * p], b = ((const float4 *)out)[2 * p + 1];
+            const float o[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-            for (int e = 0; e < 8; e++) {
-                const int k = ch + e;
-                if (k < nf) {
-                    const float d = out[p * out_cs + k] - target[p * nf + k];
-                    acc += (double)d * (double)d;
-                    g[e] = (float)(2.0 * inv_count) * d;
-                } else {
-                    g[e] = 0.0f;
-                }
+            for (int k = 0; k < 8; k++)
+                if (k < nf)
+                    d[k] = o[k] - target[p * nf + k];
+        }
+        float gr[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            gr[k] = scale * d[k];
+            if (fabsf(d[k]) < 1e12f) {
+                const float sq = __fmul_rn(d[k], d[k]);
+                add(sq, __fmaf_rn(d[k], d[k], -sq));
+            } else {
+                wide += (double)d[k] * (double)d[k];
             }
-            *(uint4 *)(dout + p * c + ch) = pack8(g);
+        }
+        const uint4 mine = pack8(gr);
+        uint4 *row = (uint4 *)dout + 32 * g * cv;
+        for (int j = 0; j < cv; j++) {
+            const int q = 32 * j + lane, pix = q / cv, chunk = q - pix * cv;
+            uint4 u;
+            u.x = __shfl_sync(0xffffffffu, mine.x, pix);
+            u.y = __shfl_sync(0xffffffffu, mine.y, pix);
+            u.z = __shfl_sync(0xffffffffu, mine.z, pix);
+            u.w = __shfl_sync(0xffffffffu, mine.w, pix);
+            if (32 * g + pix < npix)
+                row[q] = chunk == 0 ? u : make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    red[threadIdx.x] = acc;
+    double s = (double)hi + (double)lo + wide;
+    for (int o = 16; o > 0; o >>= 1)
+        s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0)
+        red[w] = s;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int j = 1; j < 8; j++)
+            s += red[j];
+        partial[blockIdx.x] = s;
     }
-    if (threadIdx.x == 0)
-        partial[blockIdx.x] = red[0];
 }
 
 // Adam (Kingma and Ba, Algorithm 1) on FP32 master parameters; omb1 = 1 - beta1,
@@ -876,6 +988,7 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
                             float *__restrict__ v, long long count, float lr, float beta1, float beta2, float omb1,
                             float omb2, float eps, float c1, float c2)
 {
+    grid_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x) {
         const float gi = g[i];
@@ -892,6 +1005,7 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
 __global__ void weights_to_bf16_kernel(const float *__restrict__ w, int cout, int cin, bf16 *__restrict__ wf,
                                        bf16 *__restrict__ wd)
 {
+    grid_begin();
     const long long total = (long long)cout * 9 * cin;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
