@@ -210,6 +210,33 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
     return CNO_OK;
 }
 
+// Tiles of 8 x 16 pixels that conv64_kernel may need for one tile of 128 pixels of
+// conv_fprop_kernel and still be the faster one (flat images fill its tiles badly).
+constexpr double CONV64_TILES = 1.4;
+
+template <int BN, bool SLOPE>
+static cno_status launch_conv64(const void *in, const void *wmat, const void *slope_src, const cnok::ConvArgs &a,
+                                cudaStream_t st)
+{
+    using S = cnok::Conv64Shape<BN, SLOPE>;
+    static bool attr = false;
+    if (!attr) {
+        CK(cudaFuncSetAttribute(cnok::conv64_kernel<BN, SLOPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
+        attr = true;
+    }
+    CUtensorMap mx, mw, mo, ms;
+    CS(map_nhwc(&mx, in, a.n, a.h, a.w, 64, cnok::C64_HW, cnok::C64_HH));
+    CS(map_matrix(&mw, wmat, a.cout, 9 * 64, BN));
+    mo = ms = mx;  // not used: FP32 output, no slope
+    if (BN == 64)
+        CS(map_nhwc(&mo, a.out, a.n, a.h, a.w, a.cout, cnok::C64_W, 4));
+    if (SLOPE)
+        CS(map_nhwc(&ms, slope_src, a.n, a.h, a.w, a.cout, cnok::C64_W, cnok::C64_H));
+    const dim3 grid(std::min(a.tiles, num_sms()), BN == 64 ? a.cout / 64 : 1);
+    CK(launch(cnok::conv64_kernel<BN, SLOPE>, grid, 192, S::SMEM, st, mx, mw, mo, ms, a));
+    return CNO_OK;
+}
+
 // Common launcher of forward (epi = BIAS / BIAS_LRELU) and data-gradient
 // (epi = SLOPE / PLAIN) convolutions: out[p][o] = sum_{t,i} in[p + s_t][i] wmat[o][t][i].
 static cno_status conv_launch(const void *in, int n, int h, int w, int cin, const void *wmat, int cout, int epi,
@@ -228,10 +255,7 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
         return fail(CNO_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
     const int wt = w >= 128 ? 128 : w;
     const int ht = 128 / wt;
-    CUtensorMap mx, mw;
     const int bn = pick_bn(cout);
-    CS(map_nhwc(&mx, in, n, h, w, cin, wt, ht));
-    CS(map_matrix(&mw, wmat, cout, 9 * cin, bn));
     cnok::ConvArgs a;
     a.n = n;
     a.h = h;
@@ -259,6 +283,25 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
     const long long tiles = (long long)n * a.tiles_w * a.tiles_h;
     if (tiles > 0x7fffffffLL)
         return fail(CNO_ERR_INVALID_ARG, "too many tiles");
+    const bool head = out_f32 && n_store <= 16 && cout == 64;
+    const bool plain = !out_f32 && n_store == cout && out_cs == cout;
+    if (cin == 64 && bn == 64 && (head || plain) && (epi != cnok::EPI_SLOPE || !((uintptr_t)slope_src & 15))) {
+        cnok::ConvArgs b = a;
+        b.tiles_w = (w + cnok::C64_W - 1) / cnok::C64_W;
+        b.tiles_h = (h + cnok::C64_H - 1) / cnok::C64_H;
+        const long long t64 = (long long)n * b.tiles_w * b.tiles_h;
+        if (t64 <= CONV64_TILES * tiles && t64 <= 0x7fffffffLL) {
+            b.tiles = (int)t64;
+            if (head)
+                return launch_conv64<16, false>(in, wmat, nullptr, b, st);
+            if (epi == cnok::EPI_SLOPE)
+                return launch_conv64<64, true>(in, wmat, slope_src, b, st);
+            return launch_conv64<64, false>(in, wmat, nullptr, b, st);
+        }
+    }
+    CUtensorMap mx, mw;
+    CS(map_nhwc(&mx, in, n, h, w, cin, wt, ht));
+    CS(map_matrix(&mw, wmat, cout, 9 * cin, bn));
     switch (bn) {
     case 256: return launch_fprop_bn<256>(mx, mw, a, (int)tiles, st);
     case 128: return launch_fprop_bn<128>(mx, mw, a, (int)tiles, st);

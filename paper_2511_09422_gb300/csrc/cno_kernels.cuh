@@ -492,6 +492,295 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
 }
 
 // --------------------------------------------------------------------------
+// The same convolutions for 64 input channels (the full-resolution layers).  K is
+// only 576, so conv_fprop_kernel moves 24 KB from L2 for every 128 x 64 x 64 step
+// (each input pixel nine times, the weights once per tile) and is bound by that:
+// 92 us for 1024^2 pixels, the tensor pipe 31 % active.  Here
+//   - the weights (nine taps of BN x 64, 72 KB at BN = 64) stay in shared memory;
+//   - a tile is 8 x 16 pixels and its input with the halo, 10 x 18 pixels, is one TMA
+//     box of 23 KB.  Tap (dy, dx) is the same box read from pixel (dx, dy): the eight
+//     pixels of an image row are one 8-row group of the operand (128 bytes a
+//     pixel, swizzled by their address), and the groups lie 10 pixels (1280 bytes)
+//     apart.  24 KB a tile instead of 216 KB;
+//   - bf16 results go through shared memory and leave by TMA, one box of 8 x 4 pixels
+//     per epilogue warp, and the activations whose slope multiplies a data gradient
+//     come in by TMA: whole lines both ways, no masks.
+// One persistent CTA per SM: TMA warp, MMA warp, four epilogue warps, two
+// accumulators.  The taps are added in the same order as in conv_fprop_kernel, so
+// the results are the same bits.  BN = 16 serves the head, of whose 64 outputs at
+// most 16 are stored.
+// --------------------------------------------------------------------------
+constexpr int C64_W = 8, C64_H = 16;              // pixels of a tile
+constexpr int C64_HW = C64_W + 2, C64_HH = C64_H + 2;
+
+template <int BN, bool SLOPE>
+struct Conv64Shape {
+    static constexpr int A_BYTES = C64_HW * C64_HH * ROW_BYTES;
+    static constexpr int A_STAGE = (A_BYTES + 1023) / 1024 * 1024;
+    static constexpr int STAGES = SLOPE ? 3 : 4;
+    static constexpr int TAP_BYTES = BN * ROW_BYTES;
+    static constexpr int TILE_BYTES = BM * ROW_BYTES;  // 128 pixels of 64 bf16 channels
+    static constexpr int OFF_A = 9 * TAP_BYTES;
+    static constexpr int OFF_OUT = OFF_A + STAGES * A_STAGE;            // two staged output tiles
+    static constexpr int OFF_SLOPE = OFF_OUT + (BN == 64 ? 2 : 0) * TILE_BYTES;  // two slope tiles
+    static constexpr int OFF_BAR = OFF_SLOPE + (SLOPE ? 2 : 0) * TILE_BYTES;
+    static constexpr int SMEM = OFF_BAR + 256 + BN * 4 + 1024 /* alignment */;
+    static constexpr int TMEM_COLS = 2 * BN;
+};
+
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void *src, int c0, int c1, int c2, int c3)
+{
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                     (uint64_t)map),
+                 "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(src))
+                 : "memory");
+}
+
+// 16 consecutive FP32 columns of the warp's 32 tensor-memory lanes.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; i++)
+        v[i] = __uint_as_float(r[i]);
+}
+
+template <int BN, bool SLOPE>
+__global__ void __launch_bounds__(192, 1)
+    conv64_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
+                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_slope,
+                  const ConvArgs a)
+{
+    using S = Conv64Shape<BN, SLOPE>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *full = (uint64_t *)(smem + S::OFF_BAR);
+    uint64_t *empty = full + S::STAGES;
+    uint64_t *w_full = empty + S::STAGES;
+    uint64_t *acc_full = w_full + 1;    // [2]
+    uint64_t *acc_empty = acc_full + 2; // [2]
+    uint64_t *sl_full = acc_empty + 2;  // [2]
+    uint64_t *sl_empty = sl_full + 2;   // [2]
+    uint32_t *tmem_holder = (uint32_t *)(sl_empty + 2);
+    volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
+    float *sbias = (float *)(smem + S::OFF_BAR + 256);
+
+    grid_begin();
+    if (*(volatile unsigned *)a.status != 0u)
+        return;  // an earlier launch failed: leave the output untouched
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = blockIdx.y * 64;
+    const bool has_bias = a.epi == EPI_BIAS || a.epi == EPI_BIAS_LRELU;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S::STAGES; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(w_full, 1);
+        for (int b = 0; b < 2; b++) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 4);
+            mbar_init(&sl_full[b], 1);
+            mbar_init(&sl_empty[b], 4);
+        }
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp >= 2 && has_bias)
+        for (int c = threadIdx.x - 64; c < BN; c += 128)
+            sbias[c] = a.bias[n0 + c];
+    if (warp == 1)
+        tmem_alloc(tmem_holder, S::TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_holder;
+
+    auto place = [&](int tile, int &w0, int &h0, int &img) {
+        const int tw = tile % a.tiles_w, r = tile / a.tiles_w;
+        w0 = tw * C64_W;
+        h0 = (r % a.tiles_h) * C64_H;
+        img = r / a.tiles_h;
+    };
+
+    if (warp == 0 && lane == 0) {
+        mbar_expect_tx(w_full, 9 * S::TAP_BYTES);
+        for (int t = 0; t < 9; t++)
+            tma_load_2d(smem + t * S::TAP_BYTES, &map_w, w_full, t * KB, n0);
+        int it = 0;
+        for (int tile = blockIdx.x; tile < a.tiles && !*abort_flag; tile += gridDim.x, it++) {
+            int w0, h0, img;
+            place(tile, w0, h0, img);
+            const int s = it % S::STAGES, use = it / S::STAGES;
+            if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1, a.status)) {
+                atomicOr(a.status, ST_TIMEOUT_PRODUCER);
+                *abort_flag = 1;
+                break;
+            }
+            mbar_expect_tx(&full[s], S::A_BYTES);
+            tma_load_4d(smem + S::OFF_A + s * S::A_STAGE, &map_x, &full[s], 0, w0 - 1, h0 - 1, img);
+            if (SLOPE) {
+                const int b = it & 1;
+                if (it >= 2 && !mbar_wait(&sl_empty[b], ((it >> 1) - 1) & 1, a.status)) {
+                    atomicOr(a.status, ST_TIMEOUT_PRODUCER);
+                    *abort_flag = 1;
+                    break;
+                }
+                mbar_expect_tx(&sl_full[b], S::TILE_BYTES);
+                tma_load_4d(smem + S::OFF_SLOPE + b * S::TILE_BYTES, &map_slope, &sl_full[b], n0, w0, h0, img);
+            }
+        }
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = idesc_bf16(BM, BN, 0, 0);
+        const uint32_t sw = smem_u32(smem);
+        int it = 0;
+        bool ok = mbar_wait(w_full, 0, a.status);
+        for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, it++) {
+            const int acc = it & 1, use = it >> 1, s = it % S::STAGES;
+            ok = !*abort_flag && (use == 0 || mbar_wait(&acc_empty[acc], (use - 1) & 1, a.status)) &&
+                 mbar_wait(&full[s], (it / S::STAGES) & 1, a.status);
+            if (!ok)
+                break;
+            tc_fence_after();
+            const uint32_t dt = tmem + (uint32_t)(acc * BN);
+            const uint32_t sa = sw + S::OFF_A + s * S::A_STAGE;
+#pragma unroll
+            for (int t = 0; t < 9; t++) {
+                // K-major, 128-byte swizzle; the k-th 16-element slice starts 32 B further in
+                const uint64_t ad = sw128_desc(sa + ((t / 3) * C64_HW + t % 3) * ROW_BYTES, 16, C64_HW * ROW_BYTES);
+                const uint64_t bd = sw128_desc(sw + t * S::TAP_BYTES, 16, 1024);
+#pragma unroll
+                for (int k = 0; k < KB / 16; k++)
+                    umma_bf16(dt, ad + 2 * k, bd + 2 * k, idesc, (t | k) != 0);
+            }
+            umma_commit(&empty[s]);
+            umma_commit(&acc_full[acc]);
+        }
+        if (!ok) {
+            atomicOr(a.status, ST_TIMEOUT_MMA);
+            *abort_flag = 1;
+        }
+    } else if (warp >= 2) {
+        const int q = warp & 3;
+        const int r = 32 * q + lane, px = r % C64_W, py = r / C64_W;
+        int it = 0;
+        for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x, it++) {
+            const int acc = it & 1, use = it >> 1;
+            // the tensor-memory loads are warp-collective: take the decision per warp
+            bool ok = mbar_wait(&acc_full[acc], use & 1, a.status);
+            if (SLOPE)
+                ok = ok && mbar_wait(&sl_full[acc], use & 1, a.status);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0)
+                    atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                break;
+            }
+            tc_fence_after();
+            int w0, h0, img;
+            place(tile, w0, h0, img);
+            const uint32_t td = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * BN);
+            if constexpr (BN == 64) {
+                // this warp's 32 pixels (8 x 4) of the staged tile; the store two tiles ago has read them
+                uint8_t *stage = smem + S::OFF_OUT + acc * S::TILE_BYTES + q * 32 * ROW_BYTES;
+                const uint8_t *slope = smem + S::OFF_SLOPE + acc * S::TILE_BYTES + r * ROW_BYTES;
+                if (lane == 0)
+                    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                __syncwarp();
+#pragma unroll
+                for (int c0 = 0; c0 < BN; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(td + (uint32_t)c0, v);
+                    if (has_bias) {
+#pragma unroll
+                        for (int i = 0; i < 32; i++) {
+                            const float z = v[i] + sbias[c0 + i];
+                            v[i] = a.epi == EPI_BIAS_LRELU ? lrelu(z) : z;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int chunk = ((c0 / 8 + j) ^ (lane & 7)) * 16;
+                        if (SLOPE) {
+                            const uint4 u = *(const uint4 *)(slope + chunk);
+                            const bf16 *yb = (const bf16 *)&u;
+#pragma unroll
+                            for (int e = 0; e < 8; e++)
+                                v[8 * j + e] *= lrelu_slope(__bfloat162float(yb[e]));
+                        }
+                        uint4 u;
+                        __nv_bfloat162 *p2 = (__nv_bfloat162 *)&u;
+#pragma unroll
+                        for (int e = 0; e < 4; e++)
+                            p2[e] = __floats2bfloat162_rn(v[8 * j + 2 * e], v[8 * j + 2 * e + 1]);
+                        *(uint4 *)(stage + lane * ROW_BYTES + chunk) = u;
+                    }
+                }
+                tc_fence_before();
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&acc_empty[acc]);
+                    if (SLOPE)
+                        mbar_arrive(&sl_empty[acc]);
+                    if (h0 + 4 * q < a.h)
+                        tma_store_4d(&map_out, stage, n0, w0, h0 + 4 * q, img);
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+            } else {
+                float v[16];
+                tmem_ld16(td, v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&acc_empty[acc]);
+                if (w0 + px < a.w && h0 + py < a.h) {
+                    const long long pix = ((long long)img * a.h + h0 + py) * a.w + w0 + px;
+#pragma unroll
+                    for (int i = 0; i < 16; i++) {
+                        const float z = v[i] + (has_bias ? sbias[i] : 0.0f);
+                        v[i] = a.epi == EPI_BIAS_LRELU ? lrelu(z) : z;
+                    }
+                    float *o = (float *)a.out + pix * a.out_cs;
+                    if (a.n_store == 8 && (a.out_cs & 3) == 0) {
+                        ((float4 *)o)[0] = make_float4(v[0], v[1], v[2], v[3]);
+                        ((float4 *)o)[1] = make_float4(v[4], v[5], v[6], v[7]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; i++)
+                            if (i < a.n_store)
+                                o[i] = v[i];
+                    }
+                    if (a.out2) {
+                        float *o2 = a.out2 + pix * a.out2_cs;
+#pragma unroll
+                        for (int i = 0; i < 8; i++)
+                            if (i < a.n2)
+                                o2[i] = v[i];
+                    }
+                }
+            }
+        }
+        if (BN == 64 && lane == 0)
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, S::TMEM_COLS);
+    }
+}
+
+// --------------------------------------------------------------------------
 // Weight gradient of one tap: D[o][i] = sum_p dz[p][o] x[p + s_tap][i] over a
 // range of 64-pixel K blocks.  Both operands are loaded from the NHWC tensors
 // as they are, so they are MN-major (the 64 channels of one pixel form one

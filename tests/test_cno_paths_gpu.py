@@ -52,3 +52,50 @@ def test_loss_is_the_mean_square_in_fp64(n, h, w, scale):
     loss = net.train_step(x, t, 0.0, update=False)
     assert loss == pytest.approx(float((d * d).mean()), rel=1e-12)
     net.close()
+
+
+def _conv_case(n, h, w, cin, cout, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn((n, h, w, cin), device="cuda", generator=gen).to(torch.bfloat16)
+    w32 = torch.randn((cout, 9, cin), device="cuda", generator=gen) / (9 * cin) ** 0.5
+    b = torch.randn(cout, device="cuda", generator=gen)
+    return x, w32, b
+
+
+def _ref(x, w, b=None):
+    """FP64 convolution and the sum of its terms' magnitudes (NHWC)."""
+    def conv(v, k, c):
+        o, _, i = k.shape
+        z = torch.nn.functional.conv2d(v.double().permute(0, 3, 1, 2), k.double().reshape(o, 3, 3, i).permute(0, 3, 1, 2), c, padding=1)
+        return z.permute(0, 2, 3, 1)
+    return conv(x, w, None if b is None else b.double()), conv(x.abs(), w.abs(), None if b is None else b.double().abs())
+
+
+def _inside(got, ref, mag, what):
+    tol = 2.0 ** -8 * ref.abs() + 2.0 ** -12 * mag + 1e-30
+    bad = (got.double() - ref).abs() > tol
+    assert not bool(bad.any()), "%s: %d of %d outside the bar" % (what, int(bad.sum()), bad.numel())
+
+
+# 64 input channels: tiles of 8 x 16 pixels with whole, ragged and single tiles, several per block, three output blocks
+@pytest.mark.parametrize("n,h,w,cout", [(1, 1, 1, 64), (1, 16, 8, 64), (2, 17, 16, 64), (1, 15, 256, 64), (1, 33, 129, 64),
+                                        (3, 64, 64, 64), (2, 48, 130, 192), (5, 128, 128, 64)])
+def test_64_channel_layers(n, h, w, cout):
+    from paper_2511_09422_gb300 import cno
+    x, w32, b = _conv_case(n, h, w, 64, cout, h + w)
+    wf, wd = cno.weights_to_bf16(w32)
+    ref, mag = _ref(x, wf, b)
+    for act in (True, False):
+        want = torch.where(ref > 0, ref, ref / 16) if act else ref
+        _inside(cno.conv3x3_forward(x, wf, b, act), want, mag, "forward")
+    if cout == 64:
+        y = cno.conv3x3_forward(x, wf, b, False, out_f32=True, n_store=8)
+        assert bool(((y.double() - ref[..., :8]).abs() <= 2.0 ** -12 * mag[..., :8] + 1e-30).all())
+    # data gradient: 64 channels in, cin out
+    dz, w32, _ = _conv_case(n, h, w, 64, cout, h + w + 1)  # weights [cout][9][64] read as Wd
+    wd = w32.to(torch.bfloat16)
+    slope = torch.randn((n, h, w, cout), device="cuda").to(torch.bfloat16)
+    ref, mag = _ref(dz, wd)
+    _inside(cno.conv3x3_dgrad(dz, wd), ref, mag, "dgrad")
+    k = torch.where(slope > 0, 1.0, 1.0 / 16).double()
+    _inside(cno.conv3x3_dgrad(dz, wd, slope), ref * k, mag * k, "dgrad with slope")
