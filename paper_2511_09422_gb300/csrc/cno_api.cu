@@ -324,6 +324,20 @@ static cno_status launch_wgrad_bn(const CUtensorMap &mdz, const CUtensorMap &mx,
     return CNO_OK;
 }
 
+template <int G>
+static cno_status launch_wgrad64(const CUtensorMap &mdz, const CUtensorMap &mx, const cnok::WgradArgs &a,
+                                 cudaStream_t st)
+{
+    using S = cnok::Wgrad64Shape<G>;
+    static bool attr = false;
+    if (!attr) {
+        CK(cudaFuncSetAttribute(cnok::wgrad64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
+        attr = true;
+    }
+    CK(launch(cnok::wgrad64_kernel<G>, dim3(3 * (a.cout / 64), a.splits), 192, S::SMEM, st, mdz, mx, a));
+    return CNO_OK;
+}
+
 static unsigned grid_for(long long n, int block)
 {
     long long g = (n + block - 1) / block;
@@ -331,10 +345,16 @@ static unsigned grid_for(long long n, int block)
     return (unsigned)std::max(1LL, std::min(g, cap));
 }
 
+// Whether wgrad64_kernel takes a weight gradient: 64 input channels, and rows of
+// at least 8 pixels (an 8-row group of its operands lies in one image row).
+static bool use_wgrad64(int w, int cin) { return cin == 64 && w >= 8; }
+
 // Tiling of a weight gradient: 64-pixel K blocks (wt x ht pixels of one
 // image), 9 taps x output-channel tiles x input-channel tiles, and as many
 // pixel ranges ("splits") as fill one wave of two CTAs per SM, with at least
-// 8 K blocks each.
+// 8 K blocks each.  wgrad64_kernel keeps the same ranges with a third of the CTAs:
+// the tensor cores round their running sums towards zero, so the length of a range
+// is part of the result's accuracy (1.5 times the ranges moved dW by 2.4e-5).
 static void wgrad_plan(int n, int h, int w, int cin, int cout, cnok::WgradArgs *a, int *bn)
 {
     *bn = pick_bn(cin);
@@ -391,14 +411,22 @@ static cno_status wgrad_launch(const void *dz, const void *x, int n, int h, int 
     int bn;
     wgrad_plan(n, h, w, cin, cout, &a, &bn);
     CUtensorMap mdz, mx;
-    CS(map_nhwc(&mdz, dz, n, h, w, cout, a.wt, a.ht));
-    CS(map_nhwc(&mx, x, n, h, w, cin, a.wt, a.ht));
+    const bool w64 = use_wgrad64(w, cin);
+    CS(map_nhwc(&mdz, dz, n, h, w, cout, a.wt + w64, a.ht));
+    CS(map_nhwc(&mx, x, n, h, w, cin, a.wt + w64, a.ht));
     a.partial = partial;
     a.status = status;
-    switch (bn) {
-    case 256: CS(launch_wgrad_bn<256>(mdz, mx, a, st)); break;
-    case 128: CS(launch_wgrad_bn<128>(mdz, mx, a, st)); break;
-    default: CS(launch_wgrad_bn<64>(mdz, mx, a, st)); break;
+    if (w64) {
+        if (3 * (cout / 64) * a.splits <= num_sms())
+            CS(launch_wgrad64<4>(mdz, mx, a, st));
+        else
+            CS(launch_wgrad64<2>(mdz, mx, a, st));
+    } else {
+        switch (bn) {
+        case 256: CS(launch_wgrad_bn<256>(mdz, mx, a, st)); break;
+        case 128: CS(launch_wgrad_bn<128>(mdz, mx, a, st)); break;
+        default: CS(launch_wgrad_bn<64>(mdz, mx, a, st)); break;
+        }
     }
     const long long count = (long long)cout * 9 * cin;
     CK(launch(cnok::sum_partials_kernel, grid_for(count, 256), 256, 0, st, partial, a.splits, count, dw));

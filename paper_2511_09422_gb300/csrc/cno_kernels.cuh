@@ -949,6 +949,181 @@ __global__ void __launch_bounds__(192, 1)
     }
 }
 
+// --------------------------------------------------------------------------
+// Weight gradient for 64 input channels, three taps of one image row offset dy at a
+// time.  An MMA with M = 128 reads its A operand for about 64 cycles per 16 pixels
+// whatever N <= 128 is, and conv_wgrad_kernel spends one on each tap, half of M
+// empty at 64 output channels, loading 16 KB of pixels for four of them: 160 us for 16 x 256^2,
+// 480 TFLOP/s.  Here M = 128 holds x at two column offsets a, N = 128 holds dz at
+// two column offsets b, and the tap is dx = a - b:
+//   D[(a, i)][(b, o)] = sum_p x[p + a + dy][i] dz[p + b][o],  a, b in {-1, 0}
+//   (-1, 0): dx = -1;  (0, 0): dx = 0;  (0, -1): dx = +1;  (-1, -1): dx = 0 again, not used.
+// Both offsets are the same staged pixels read one 128-byte row further on (the
+// leading-dimension offset of the operands).  dz[-1] is the zero fill of the
+// load, and the one pixel pair per row that no block holds, x[w] dz[w-1], is zero.
+// A K block is 64 pixels: wt x ht of one image, loaded with one column more.
+// Partials per pixel range as in conv_wgrad_kernel: [split][o][9 cin].
+// --------------------------------------------------------------------------
+// A stage is G K blocks: waiting for a stage and committing it costs the issuing
+// thread some 250 cycles, an MMA 70 (at one block a stage, 148 us for 16 x 256^2; with
+// half the loads, or with twice the stages, as long).  G = 4 where the CTAs fit
+// one per SM, else G = 2 and two per SM.
+template <int G>
+struct Wgrad64Shape {
+    static constexpr int SLOT = 9 * 1024;  // (wt + 1) ht <= 72 pixels of 128 bytes
+    static constexpr int BLOCK = 2 * SLOT; // x, then dz
+    static constexpr int STAGE = G * BLOCK;
+    static constexpr int STAGES = 3;
+    static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
+    static constexpr int TMEM_COLS = 128;
+};
+
+template <int G>
+__global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
+    wgrad64_kernel(const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_x,
+                   const WgradArgs a)
+{
+    using S = Wgrad64Shape<G>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *full = (uint64_t *)(smem + S::STAGES * S::STAGE);
+    uint64_t *empty = full + S::STAGES;
+    uint64_t *done = empty + S::STAGES;
+    uint32_t *tmem_holder = (uint32_t *)(done + 1);
+    volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
+
+    grid_begin();
+    if (*(volatile unsigned *)a.status != 0u)
+        return;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int dy = (int)(blockIdx.x % 3) - 1, o0 = (int)(blockIdx.x / 3) * 64;
+    const int split = blockIdx.y;
+    const int kb_lo = split * a.kb_per_split;
+    const int nk = min(a.kb_total, kb_lo + a.kb_per_split) - kb_lo;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S::STAGES; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1)
+        tmem_alloc(tmem_holder, S::TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_holder;
+    const int pitch = (a.wt + 1) * ROW_BYTES;  // bytes of a staged image row
+
+    // The two issuing threads keep their positions instead of dividing for them (which
+    // took longer than a block's MMAs).
+    if (warp == 0 && lane == 0) {
+        const uint32_t bytes = 2 * pitch * a.ht;
+        int tw = kb_lo % a.tiles_w, th = kb_lo / a.tiles_w % a.tiles_h, img = kb_lo / a.tiles_w / a.tiles_h;
+        int s = 0, phase = 1;  // the parity of an empty slot's first wait is passed at once
+        for (int j = 0; j < nk; j += G) {
+            if (!mbar_wait(&empty[s], phase, a.status)) {
+                atomicOr(a.status, ST_TIMEOUT_PRODUCER);
+                *abort_flag = 1;
+                break;
+            }
+            uint8_t *st = smem + s * S::STAGE;
+            const int blocks = min(G, nk - j);
+            mbar_expect_tx(&full[s], blocks * bytes);
+            for (int g = 0; g < blocks; g++, st += S::BLOCK) {
+                const int pw = tw * a.wt, ph = th * a.ht;
+                tma_load_4d(st, &map_x, &full[s], 0, pw - 1, ph + dy, img);
+                tma_load_4d(st + S::SLOT, &map_dz, &full[s], o0, pw - 1, ph, img);
+                if (++tw == a.tiles_w) {
+                    tw = 0;
+                    if (++th == a.tiles_h) {
+                        th = 0;
+                        img++;
+                    }
+                }
+            }
+            if (++s == S::STAGES) {
+                s = 0;
+                phase ^= 1;
+            }
+        }
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = idesc_bf16(BM, 128, 1, 1);
+        // 16 pixels per MMA: of one image row, or (wt = 8) eight of two rows each
+        const uint32_t sbo = a.wt >= 16 ? 1024 : pitch;
+        // MN-major, 128-byte swizzle: the two 64-channel halves are one pixel (128 B) apart
+        const uint64_t base = sw128_desc(smem_u32(smem), ROW_BYTES, sbo);
+        uint32_t off[4];  // of the block's k-th 16 pixels, in the descriptor's 16-byte units
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            off[k] = (16 * k / a.wt * pitch + 16 * k % a.wt * ROW_BYTES) >> 4;
+        int s = 0, phase = 0;
+        bool ok = true;
+        for (int j = 0; j < nk; j += G) {
+            if (!mbar_wait(&full[s], phase, a.status)) {
+                atomicOr(a.status, ST_TIMEOUT_MMA);
+                *abort_flag = 1;
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                if (j + g >= nk)
+                    break;
+                const uint64_t at = base + (uint64_t)((s * S::STAGE + g * S::BLOCK) >> 4);
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    umma_bf16(tmem, at + off[k], at + off[k] + (S::SLOT >> 4), idesc, (j | g | k) != 0);
+            }
+            umma_commit(&empty[s]);
+            if (++s == S::STAGES) {
+                s = 0;
+                phase ^= 1;
+            }
+        }
+        if (ok && nk > 0)
+            umma_commit(done);
+    } else if (warp >= 2) {
+        const int q = warp & 3;
+        const int i = 32 * (q & 1) + lane;  // input channel; q / 2: column offset a + 1 of x
+        const int ldk = 9 * 64, tap0 = 3 * (dy + 1);
+        float *dst = a.partial + ((long long)split * a.cout + o0) * ldk + i;
+        const bool have = nk > 0;
+        const bool ok = !have || __all_sync(0xffffffffu, mbar_wait(done, 0, a.status));
+        if (!ok) {
+            if (lane == 0)
+                atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+        } else {
+            tc_fence_after();
+#pragma unroll 1
+            for (int c0 = 0; c0 < 128; c0 += 32) {
+                // columns (b + 1, o): b = -1 in 0 .. 63, b = 0 in 64 .. 127
+                const int dx = (q >> 1) - (c0 >> 6);  // a - b
+                if (c0 < 64 && q < 2)
+                    continue;  // (-1, -1)
+                float v[32];
+                if (have)
+                    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+                float *d = dst + (long long)(c0 & 63) * ldk + (tap0 + dx + 1) * 64;
+#pragma unroll
+                for (int e = 0; e < 32; e++)
+                    d[(long long)e * ldk] = have ? v[e] : 0.0f;
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, S::TMEM_COLS);
+    }
+}
+
 __device__ __forceinline__ void unpack8(uint4 u, float (&f)[8])
 {
     const __nv_bfloat162 *p = (const __nv_bfloat162 *)&u;

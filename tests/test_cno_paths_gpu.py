@@ -99,3 +99,23 @@ def test_64_channel_layers(n, h, w, cout):
     _inside(cno.conv3x3_dgrad(dz, wd), ref, mag, "dgrad")
     k = torch.where(slope > 0, 1.0, 1.0 / 16).double()
     _inside(cno.conv3x3_dgrad(dz, wd, slope), ref * k, mag * k, "dgrad with slope")
+
+
+# 64 input channels: K blocks of one row, of two, four and eight rows (w 64 .. 8), ragged rows, widths the kernel leaves
+# to the general one (4), one block, several pixel ranges, several output tiles
+@pytest.mark.parametrize("n,h,w,cout", [(1, 1, 8, 64), (2, 5, 4, 64), (1, 8, 8, 64), (3, 9, 16, 128), (1, 33, 32, 64),
+                                        (2, 40, 64, 64), (1, 7, 129, 192), (2, 31, 200, 256), (4, 128, 128, 64)])
+def test_64_channel_weight_gradients(n, h, w, cout):
+    from paper_2511_09422_gb300 import cno
+    x, _, _ = _conv_case(n, h, w, 64, cout, 3 * h + w)
+    dz = torch.randn((n, h, w, cout), device="cuda").to(torch.bfloat16)
+    dw, db = cno.conv3x3_wgrad(dz, x)
+
+    def ref(d, v):
+        vp = torch.nn.functional.pad(v.double(), (0, 0, 1, 1, 1, 1))
+        taps = [torch.einsum("nhwo,nhwi->oi", d.double(), vp[:, dy:dy + h, dx:dx + w]) for dy in range(3) for dx in range(3)]
+        return torch.stack(taps, 1)
+
+    assert bool(((dw.double() - ref(dz, x)).abs() <= 2.0 ** -13 * ref(dz.abs(), x.abs()) + 1e-30).all())
+    s = dz.double().sum((0, 1, 2))
+    assert bool(((db.double() - s).abs() <= 2.0 ** -13 * dz.double().abs().sum((0, 1, 2)) + 1e-30).all())
