@@ -239,10 +239,11 @@ static cno_status launch_conv64(const void *in, const void *wmat, const void *sl
 
 // Common launcher of forward (epi = BIAS / BIAS_LRELU) and data-gradient
 // (epi = SLOPE / PLAIN) convolutions: out[p][o] = sum_{t,i} in[p + s_t][i] wmat[o][t][i].
+// nonzero > 0: the caller knows the input channels from there on to be zero.
 static cno_status conv_launch(const void *in, int n, int h, int w, int cin, const void *wmat, int cout, int epi,
                               const float *bias, const void *slope_src, void *out, int out_f32, int out_cs,
                               int n_store, unsigned *status, cudaStream_t st, float *out2 = nullptr, int out2_cs = 0,
-                              int n2 = 0)
+                              int n2 = 0, int nonzero = 0)
 {
     CS(check_image(n, h, w));
     if (!chan_ok(cin) || !chan_ok(cout))
@@ -276,6 +277,7 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
     a.out_cs = out_cs;
     a.n_store = n_store;
     a.out_f32 = out_f32;
+    a.ksteps = nonzero > 0 && nonzero <= 48 ? (nonzero + 15) / 16 : 4;
     a.out2 = out2;
     a.out2_cs = out2_cs;
     a.n2 = n2;
@@ -378,11 +380,12 @@ static void wgrad_plan(int n, int h, int w, int cin, int cout, cnok::WgradArgs *
     a->splits = (a->kb_total + a->kb_per_split - 1) / a->kb_per_split;
 }
 
-// Blocks of the bias-gradient first pass: two per SM, at least 256 pixels each.
+// Blocks of the bias-gradient first pass: four per SM (with two, 31 us for 134 MB), at
+// least 256 pixels each.
 static int bias_blocks(int n, int h, int w)
 {
     const long long npix = (long long)n * h * w;
-    return (int)std::max(1LL, std::min((long long)2 * num_sms(), (npix + 255) / 256));
+    return (int)std::max(1LL, std::min((long long)4 * num_sms(), (npix + 255) / 256));
 }
 
 // FP32 scratch of a weight gradient: the per-range partials of dW, reused for
@@ -519,13 +522,26 @@ extern "C" cno_status cno_wait_selftest(double seconds, int *gave_up, double *el
     return CNO_OK;
 }
 
+// One more layer of a weight conversion: a block for every 1024 weights.
+static void add_weights(cnok::WeightLayers *a, const float *w, int cout, int cin, void *wf, void *wd)
+{
+    const int l = a->n++;
+    const long long total = (long long)cout * 9 * cin;
+    a->w[l] = w;
+    a->cout[l] = cout;
+    a->cin[l] = cin;
+    a->wf[l] = (bf16 *)wf;
+    a->wd[l] = (bf16 *)wd;
+    a->block0[l + 1] = a->block0[l] + (int)std::min((total + 1023) / 1024, (long long)num_sms() * 8);
+}
+
 extern "C" cno_status cno_weights_to_bf16(const float *w, int cout, int cin, void *wf, void *wd, void *stream)
 {
     if (!w || !wf || !wd || cout < 1 || cin < 1)
         return fail(CNO_ERR_INVALID_ARG, "bad weight conversion arguments");
-    const long long total = (long long)cout * 9 * cin;
-    CK(launch(cnok::weights_to_bf16_kernel, grid_for(total, 256), 256, 0, (cudaStream_t)stream, w, cout, cin, (bf16 *)wf,
-              (bf16 *)wd));
+    cnok::WeightLayers a = {};
+    add_weights(&a, w, cout, cin, wf, wd);
+    CK(launch(cnok::weights_to_bf16_kernel, a.block0[1], 256, 0, (cudaStream_t)stream, a));
     return CNO_OK;
 }
 
@@ -768,10 +784,13 @@ extern "C" cno_status cno_num_params(const cno_net *net, long long *out)
 
 static cno_status refresh_bf16(cno_net *net)
 {
+    cnok::WeightLayers a = {};
+    static_assert(cnok::MAX_LAYERS >= 12, "a network has twelve layers");
     for (int k = 0; k < 12; k++) {
         const Layer &L = net->layers[k];
-        CS(cno_weights_to_bf16(net->p + L.w_off, L.cout, L.cin, net->wf[k], net->wd[k], net->st));
+        add_weights(&a, net->p + L.w_off, L.cout, L.cin, net->wf[k], net->wd[k]);
     }
+    CK(launch(cnok::weights_to_bf16_kernel, a.block0[12], 256, 0, net->st, a));
     return CNO_OK;
 }
 
@@ -910,7 +929,7 @@ static cno_status dgrad(cno_net *net, int k, const bf16 *dz, int lv, const bf16 
     const Layer &L = net->layers[k];
     return conv_launch(dz, net->an, net->ah >> lv, net->aw >> lv, L.cout, net->wd[k], L.cin,
                        slope_src ? cnok::EPI_SLOPE : cnok::EPI_PLAIN, nullptr, slope_src, dx, 0, L.cin, L.cin,
-                       net->status, net->st);
+                       net->status, net->st, nullptr, 0, 0, k == 11 ? net->nf : 0);  // the loss has nf channels
 }
 
 static cno_status wgrad(cno_net *net, int k, const bf16 *dz, const bf16 *x, int lv)

@@ -246,6 +246,7 @@ struct ConvArgs {
     const bf16 *slope_src;      // EPI_SLOPE: y whose lrelu slope multiplies the result (NHWC, cout channels)
     void *out;                  // NHWC, out_cs channels per pixel
     int out_cs, n_store, out_f32;
+    int ksteps;                 // conv64_kernel: 16-channel steps of a tap that can be non-zero (4: all)
     float *out2;                // FP32 outputs only: the first n2 <= min(8, n_store) channels again, out2_cs per pixel
     int out2_cs, n2;
     unsigned *status;
@@ -660,7 +661,8 @@ __global__ void __launch_bounds__(192, 1)
                 const uint64_t bd = sw128_desc(sw + t * S::TAP_BYTES, 16, 1024);
 #pragma unroll
                 for (int k = 0; k < KB / 16; k++)
-                    umma_bf16(dt, ad + 2 * k, bd + 2 * k, idesc, (t | k) != 0);
+                    if (k < a.ksteps)
+                        umma_bf16(dt, ad + 2 * k, bd + 2 * k, idesc, (t | k) != 0);
             }
             umma_commit(&empty[s]);
             umma_commit(&acc_full[acc]);
@@ -1464,15 +1466,30 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
     }
 }
 
-// bf16 copies of one layer's FP32 weights W[o][t][i]: the forward matrix
-// (same layout) and the data-gradient matrix Wd[i][t][o] = W[o][8 - t][i].
-__global__ void weights_to_bf16_kernel(const float *__restrict__ w, int cout, int cin, bf16 *__restrict__ wf,
-                                       bf16 *__restrict__ wd)
+// bf16 copies of FP32 weights W[o][t][i]: the forward matrix (same layout) and the
+// data-gradient matrix Wd[i][t][o] = W[o][8 - t][i].  One launch takes the layers of
+// a network (each block works on one of them; twelve launches of a few
+// microseconds each took 51 us a training step).
+constexpr int MAX_LAYERS = 12;
+struct WeightLayers {
+    int n;
+    int block0[MAX_LAYERS + 1];  // first block of a layer
+    int cout[MAX_LAYERS], cin[MAX_LAYERS];
+    const float *w[MAX_LAYERS];
+    bf16 *wf[MAX_LAYERS], *wd[MAX_LAYERS];
+};
+
+__global__ void __launch_bounds__(256) weights_to_bf16_kernel(const __grid_constant__ WeightLayers a)
 {
     grid_begin();
-    const long long total = (long long)cout * 9 * cin;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
+    int l = 0;
+    while (l + 1 < a.n && (int)blockIdx.x >= a.block0[l + 1])
+        l++;
+    const int cout = a.cout[l], cin = a.cin[l];
+    const float *__restrict__ w = a.w[l];
+    bf16 *__restrict__ wf = a.wf[l], *__restrict__ wd = a.wd[l];
+    const long long total = (long long)cout * 9 * cin, step = (long long)(a.block0[l + 1] - a.block0[l]) * blockDim.x;
+    for (long long idx = (blockIdx.x - a.block0[l]) * (long long)blockDim.x + threadIdx.x; idx < total; idx += step) {
         const int i = (int)(idx % cin);
         const int t = (int)((idx / cin) % 9);
         const int o = (int)(idx / (9LL * cin));
