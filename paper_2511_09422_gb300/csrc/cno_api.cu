@@ -1172,6 +1172,7 @@ __global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *__
                                                                  const float *__restrict__ T, HCoef hc, int nx, int ny,
                                                                  double *__restrict__ part)
 {
+    cnok::grid_begin();
     ff sum[6];       // phi, chi, f_s, 1 - phi^2, |grad phi|, rho H
     double wide[6];  // the cells evaluated in FP64
     float lo = INFINITY, hi = -INFINITY;  // T
@@ -1272,9 +1273,11 @@ __global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *__
 __global__ void __launch_bounds__(32 * NCHK) field_total_kernel(const double *__restrict__ part, int blocks,
                                                                 double *__restrict__ out)
 {
+    cnok::grid_begin();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto join = [&](double a, double b) { return k == 5 ? fmin(a, b) : (k == 6 ? fmax(a, b) : a + b); };
     double s = k == 5 ? INFINITY : (k == 6 ? -INFINITY : 0.0);
+#pragma unroll 8
     for (int b = lane; b < blocks; b += 32) s = join(s, part[(long long)b * NCHK + k]);
     for (int o = 16; o > 0; o >>= 1) s = join(s, __shfl_down_sync(0xffffffffu, s, o));
     if (lane == 0) out[k] = s;
@@ -1351,15 +1354,68 @@ extern "C" cno_status cno_apply_update(const float *const *src, float *const *ds
     return CNO_OK;
 }
 
+// Scratch of one check: the blocks' partial sums on the device (39 KB) and the result
+// in mapped host memory, written by the last kernel.  A call holds a slot until it
+// has synchronised its stream, so a returned slot is idle and calls on several
+// threads and streams never share one; up to CHECK_SLOTS idle slots are kept per
+// device.  Allocating and freeing device memory and copying the result in every call
+// took 170 us beside 30 us of kernels.
+constexpr int CHECK_SLOTS = 4, CHECK_BLOCKS_MAX = 4 * 256;
+struct CheckSlot {
+    double *part = nullptr, *out = nullptr;
+};
+static std::mutex g_check_mu;
+static std::vector<CheckSlot> g_check_slots[64];
+
+static void check_slot_free(CheckSlot &s)
+{
+    cudaFree(s.part);
+    cudaFreeHost(s.out);
+    s = CheckSlot();
+}
+
+static cno_status check_slot_take(int dev, CheckSlot *s)
+{
+    {
+        std::lock_guard<std::mutex> lk(g_check_mu);
+        if (!g_check_slots[dev].empty()) {
+            *s = g_check_slots[dev].back();
+            g_check_slots[dev].pop_back();
+            return CNO_OK;
+        }
+    }
+    cudaError_t e = cudaMalloc((void **)&s->part, (size_t)CHECK_BLOCKS_MAX * NCHK * sizeof(double));
+    if (e == cudaSuccess)
+        e = cudaHostAlloc((void **)&s->out, NCHK * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess)
+        check_slot_free(*s);
+    CK(e);
+    return CNO_OK;
+}
+
+static void check_slot_return(int dev, CheckSlot &s)
+{
+    {
+        std::lock_guard<std::mutex> lk(g_check_mu);
+        if ((int)g_check_slots[dev].size() < CHECK_SLOTS) {
+            g_check_slots[dev].push_back(s);
+            return;
+        }
+    }
+    check_slot_free(s);
+}
+
 extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const float *T, const float *hcoef,
                                        int nx, int ny, double out[8], void *stream)
 {
     if (!phi || !out || nx < 1 || ny < 1)
         return fail(CNO_ERR_INVALID_ARG, "bad check arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    const int blocks = std::min(ny, 4 * num_sms());
-    double *part = nullptr;
-    CK(cudaMallocAsync(&part, (size_t)(blocks + 1) * NCHK * sizeof(double), st));
+    const int blocks = std::min(std::min(ny, 4 * num_sms()), CHECK_BLOCKS_MAX);
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64)
+        return fail(CNO_ERR_UNSUPPORTED, "device index out of range");
     HCoef hc = {0, 0, 0, 0, 0, 0};
     if (hcoef && fs && T) {
         hc = {hcoef[0], hcoef[1], hcoef[2], hcoef[3], 1, 0};
@@ -1367,15 +1423,21 @@ extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const 
             if (!(std::fabs(hcoef[k]) < DIRECT))
                 hc.wide = 1;
     }
-    field_sums_kernel<<<blocks, CHK_THREADS, 0, st>>>(phi, fs, T, hc, nx, ny, part + NCHK);
-    field_total_kernel<<<1, 32 * NCHK, 0, st>>>(part + NCHK, blocks, part);
-    cudaError_t e = cudaGetLastError();
+    CheckSlot slot;
+    CS(check_slot_take(dev, &slot));
+    cudaError_t e = launch(field_sums_kernel, blocks, CHK_THREADS, 0, st, phi, fs, T, hc, nx, ny, slot.part);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, part, NCHK * sizeof(double), cudaMemcpyDeviceToHost, st);
-    const cudaError_t fe = cudaFreeAsync(part, st);
+        e = launch(field_total_kernel, 1, 32 * NCHK, 0, st, slot.part, blocks, slot.out);
+    const cudaError_t se = cudaStreamSynchronize(st);
+    if (e == cudaSuccess)
+        e = se;
+    if (e == cudaSuccess)
+        memcpy(out, slot.out, NCHK * sizeof(double));
+    if (se == cudaSuccess)
+        check_slot_return(dev, slot);
+    else
+        check_slot_free(slot);  // the stream is in an error state
     CK(e);
-    CK(fe);
-    CK(cudaStreamSynchronize(st));
     if (!T)
         out[5] = out[6] = 0.0;
     return CNO_OK;

@@ -151,3 +151,29 @@ def test_pack_fields_rounds_and_pads(nx, ny, cin, nfield):
         want[0, ..., k] = ((f[k] - float(off[k])) * float(sc[k])).to(torch.bfloat16)
     assert torch.equal(x, want)
     assert bool((buf[ny * nx * cin:] == 3.0).all())
+
+
+def test_field_checks_from_several_threads_and_streams():
+    """The checks keep scratch memory between calls: calls on other threads and streams give the same sums."""
+    import threading
+
+    from paper_2511_09422_gb300 import cno
+    rng = np.random.default_rng(2)
+    fields = [tuple(torch.as_tensor(rng.uniform(0, 1, (200 + 10 * i, 300)).astype(np.float32)).cuda() for _ in range(3)) for i in range(4)]
+    hc = (1.0, 0.9, 0.4, 11.0)
+    want = [cno.field_checks(*f, hc) for f in fields]
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(50):
+                if cno.field_checks(*fields[i], hc) != want[i]:
+                    bad.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
