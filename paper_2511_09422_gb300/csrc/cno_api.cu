@@ -210,9 +210,12 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
     return CNO_OK;
 }
 
-// Tiles of 8 x 16 pixels that conv64_kernel may need for one tile of 128 pixels of
-// conv_fprop_kernel and still be the faster one (flat images fill its tiles badly).
-constexpr double CONV64_TILES = 1.4;
+// Which kernel takes a convolution: 64 -> 64, 192 channels (and the FP32 head) conv64_kernel,
+// 64 or 128 -> 128, 256 conv_halo_kernel, others conv_fprop_kernel, and all of
+// them where the tiles of 8 x 16 pixels are badly filled: HALO_TILES is the number
+// of them per tile of 128 pixels in a row up to which the first two are the faster ones
+// (at one row of pixels, sixteen to one, they compute mostly padding).
+constexpr double HALO_TILES = 1.4;
 
 template <int BN, bool SLOPE>
 static cno_status launch_conv64(const void *in, const void *wmat, const void *slope_src, const cnok::ConvArgs &a,
@@ -235,6 +238,38 @@ static cno_status launch_conv64(const void *in, const void *wmat, const void *sl
     const dim3 grid(std::min(a.tiles, num_sms()), BN == 64 ? a.cout / 64 : 1);
     CK(launch(cnok::conv64_kernel<BN, SLOPE>, grid, 192, S::SMEM, st, mx, mw, mo, ms, a));
     return CNO_OK;
+}
+
+template <int CB, bool SLOPE>
+static cno_status launch_conv_halo(const void *in, const void *wmat, const void *slope_src, const cnok::ConvArgs &a,
+                                   cudaStream_t st)
+{
+    using S = cnok::ConvHaloShape<CB>;
+    static bool attr = false;
+    if (!attr) {
+        CK(cudaFuncSetAttribute(cnok::conv_halo_kernel<CB, SLOPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                S::SMEM));
+        attr = true;
+    }
+    CUtensorMap mx, mw, mo, ms;
+    CS(map_nhwc(&mx, in, a.n, a.h, a.w, a.cin, cnok::C64_HW, cnok::C64_HH));
+    CS(map_matrix(&mw, wmat, a.cout, 9 * a.cin, S::BN));
+    CS(map_nhwc(&mo, a.out, a.n, a.h, a.w, a.cout, cnok::C64_W, 4));
+    ms = mo;  // not used without slopes
+    if (SLOPE)
+        CS(map_nhwc(&ms, slope_src, a.n, a.h, a.w, a.cout, cnok::C64_W, 4));
+    const int nblocks = a.cout / S::BN;
+    const dim3 grid(std::min(a.tiles, std::max(1, num_sms() / nblocks)), nblocks);
+    CK(launch(cnok::conv_halo_kernel<CB, SLOPE>, grid, 224, S::SMEM, st, mx, mw, mo, ms, a));
+    return CNO_OK;
+}
+
+template <int CB>
+static cno_status conv_halo(const void *in, const void *wmat, const void *slope_src, const cnok::ConvArgs &a,
+                            cudaStream_t st)
+{
+    return a.epi == cnok::EPI_SLOPE ? launch_conv_halo<CB, true>(in, wmat, slope_src, a, st)
+                                    : launch_conv_halo<CB, false>(in, wmat, slope_src, a, st);
 }
 
 // Common launcher of forward (epi = BIAS / BIAS_LRELU) and data-gradient
@@ -292,13 +327,23 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
         b.tiles_w = (w + cnok::C64_W - 1) / cnok::C64_W;
         b.tiles_h = (h + cnok::C64_H - 1) / cnok::C64_H;
         const long long t64 = (long long)n * b.tiles_w * b.tiles_h;
-        if (t64 <= CONV64_TILES * tiles && t64 <= 0x7fffffffLL) {
+        if (t64 <= HALO_TILES * tiles && t64 <= 0x7fffffffLL) {
             b.tiles = (int)t64;
             if (head)
                 return launch_conv64<16, false>(in, wmat, nullptr, b, st);
             if (epi == cnok::EPI_SLOPE)
                 return launch_conv64<64, true>(in, wmat, slope_src, b, st);
             return launch_conv64<64, false>(in, wmat, nullptr, b, st);
+        }
+    }
+    if (plain && cin <= 128 && cout % 128 == 0 && (epi != cnok::EPI_SLOPE || !((uintptr_t)slope_src & 15))) {
+        cnok::ConvArgs b = a;
+        b.tiles_w = (w + cnok::C64_W - 1) / cnok::C64_W;
+        b.tiles_h = (h + cnok::C64_H - 1) / cnok::C64_H;
+        const long long th = (long long)n * b.tiles_w * b.tiles_h;
+        if (th <= HALO_TILES * tiles && th <= 0x7fffffffLL) {
+            b.tiles = (int)th;
+            return cin == 64 ? conv_halo<1>(in, wmat, slope_src, b, st) : conv_halo<2>(in, wmat, slope_src, b, st);
         }
     }
     CUtensorMap mx, mw;

@@ -783,6 +783,277 @@ __global__ void __launch_bounds__(192, 1)
 }
 
 // --------------------------------------------------------------------------
+// The same convolutions for 64 CB input channels (CB = 1, 2) and 128 output channels a
+// tile, with the weights streamed: the input tile with its halo stays in shared memory (23 KB
+// per 64 channels, read once instead of nine times), the weights come through a
+// ring of G K blocks (a K block: 64 input channels of one tap) a stage.
+// conv_fprop_kernel moves 32 KB per K block and was bound by that (600 cycles a
+// block, 54 bytes a cycle and SM from L2, where the four N = 128 MMAs take 260);
+// here it is 18.6 KB, and waiting for a stage and committing it, some 250 cycles of
+// the issuing thread, is shared by G blocks.  Results and slopes pass through shared
+// memory by TMA as in conv64_kernel, 64 channels at a time.  Same order of additions,
+// same bits.  At 512^2, before -> now (us): 64 -> 128 channels 48.7 -> 34.1, 128 -> 128 74.6 -> 65.5,
+// data gradient of 128 -> 128 with slopes 85.0 -> 66.4.  With 64 output channels a tile or four
+// input blocks (one tile buffer) it was slower than conv_fprop_kernel: 128 -> 64 50.5 -> 57.9,
+// 256 -> 256 at 256^2 57.5 -> 63.8.
+// Warps: 0 weights, 1 MMAs, 2-5 epilogue, 6 input tiles.
+// --------------------------------------------------------------------------
+template <int CB>
+struct ConvHaloShape {
+    static constexpr int BN = 128;
+    static constexpr int A_BYTES = C64_HW * C64_HH * ROW_BYTES;    // 64 channels of a tile
+    static constexpr int A_BLOCK = (A_BYTES + 1023) / 1024 * 1024;
+    static constexpr int A_BUFS = 2;
+    static constexpr int B_BLOCK = BN * ROW_BYTES;
+    static constexpr int G = CB == 1 ? 3 : 2;
+    static constexpr int B_STAGES = 3;
+    static constexpr int HALF_BYTES = BM * ROW_BYTES;              // 64 output channels of a tile
+    static constexpr int OFF_B = A_BUFS * CB * A_BLOCK;
+    static constexpr int OFF_OUT = OFF_B + B_STAGES * G * B_BLOCK; // two of them staged
+    static constexpr int OFF_BAR = OFF_OUT + 2 * HALF_BYTES;
+    static constexpr int SMEM = OFF_BAR + 256 + BN * 4 + 1024 /* alignment */;
+    static constexpr int TMEM_COLS = 2 * BN;
+    static_assert(9 * CB % G == 0, "a tile is whole stages");
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+};
+
+template <int CB, bool SLOPE>
+__global__ void __launch_bounds__(224, 1)
+    conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
+                     const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_slope,
+                     const ConvArgs a)
+{
+    using S = ConvHaloShape<CB>;
+    constexpr int BN = S::BN;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *a_full = (uint64_t *)(smem + S::OFF_BAR);  // [2]
+    uint64_t *a_empty = a_full + 2;                      // [2]
+    uint64_t *b_full = a_empty + 2;                      // [3]
+    uint64_t *b_empty = b_full + S::B_STAGES;            // [3]
+    uint64_t *acc_full = b_empty + S::B_STAGES;          // [2]
+    uint64_t *acc_empty = acc_full + 2;                  // [2]
+    uint64_t *sl_full = acc_empty + 2;                   // [4 warps][2]
+    uint32_t *tmem_holder = (uint32_t *)(sl_full + 8);
+    volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
+    float *sbias = (float *)(smem + S::OFF_BAR + 256);
+
+    grid_begin();
+    if (*(volatile unsigned *)a.status != 0u)
+        return;  // an earlier launch failed: leave the output untouched
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = blockIdx.y * BN;
+    const bool has_bias = a.epi == EPI_BIAS || a.epi == EPI_BIAS_LRELU;
+
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; b++) {
+            mbar_init(&a_full[b], 1);
+            mbar_init(&a_empty[b], 1);
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 4);
+        }
+        for (int s = 0; s < S::B_STAGES; s++) {
+            mbar_init(&b_full[s], 1);
+            mbar_init(&b_empty[s], 1);
+        }
+        for (int k = 0; k < 8; k++)
+            mbar_init(&sl_full[k], 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp >= 2 && warp < 6 && has_bias)
+        for (int c = threadIdx.x - 64; c < BN; c += 128)
+            sbias[c] = a.bias[n0 + c];
+    if (warp == 1)
+        tmem_alloc(tmem_holder, S::TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_holder;
+
+    auto place = [&](int tile, int &w0, int &h0, int &img) {
+        const int tw = tile % a.tiles_w, r = tile / a.tiles_w;
+        w0 = tw * C64_W;
+        h0 = (r % a.tiles_h) * C64_H;
+        img = r / a.tiles_h;
+    };
+    constexpr int NST = 9 * CB / S::G;  // weight stages of a tile
+
+    if (warp == 6 && lane == 0) {
+        int it = 0;
+        for (int tile = blockIdx.x; tile < a.tiles && !*abort_flag; tile += gridDim.x, it++) {
+            const int b = it % S::A_BUFS, use = it / S::A_BUFS;
+            if (use > 0 && !mbar_wait(&a_empty[b], (use - 1) & 1, a.status)) {
+                atomicOr(a.status, ST_TIMEOUT_PRODUCER);
+                *abort_flag = 1;
+                break;
+            }
+            int w0, h0, img;
+            place(tile, w0, h0, img);
+            mbar_expect_tx(&a_full[b], CB * S::A_BYTES);
+            for (int c = 0; c < CB; c++)
+                tma_load_4d(smem + (b * CB + c) * S::A_BLOCK, &map_x, &a_full[b], c * KB, w0 - 1, h0 - 1, img);
+        }
+    } else if (warp == 0 && lane == 0) {
+        int s = 0, phase = 1;  // the first wait for an empty slot passes at once
+        for (int tile = blockIdx.x; tile < a.tiles && !*abort_flag; tile += gridDim.x) {
+            for (int st = 0; st < NST; st++) {
+                if (!mbar_wait(&b_empty[s], phase, a.status)) {
+                    atomicOr(a.status, ST_TIMEOUT_PRODUCER);
+                    *abort_flag = 1;
+                    break;
+                }
+                mbar_expect_tx(&b_full[s], S::G * S::B_BLOCK);
+#pragma unroll
+                for (int g = 0; g < S::G; g++)
+                    tma_load_2d(smem + S::OFF_B + (s * S::G + g) * S::B_BLOCK, &map_w, &b_full[s],
+                                (st * S::G + g) * KB, n0);
+                if (++s == S::B_STAGES) {
+                    s = 0;
+                    phase ^= 1;
+                }
+            }
+        }
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = idesc_bf16(BM, BN, 0, 0);
+        const uint32_t sw = smem_u32(smem);
+        int it = 0, s = 0, phase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, it++) {
+            const int acc = it & 1, use = it >> 1, b = it % S::A_BUFS;
+            ok = !*abort_flag && (use == 0 || mbar_wait(&acc_empty[acc], (use - 1) & 1, a.status)) &&
+                 mbar_wait(&a_full[b], (it / S::A_BUFS) & 1, a.status);
+            const uint32_t dt = tmem + (uint32_t)(acc * BN);
+            int kb = 0;
+            for (int st = 0; ok && st < NST; st++) {
+                ok = mbar_wait(&b_full[s], phase, a.status);
+                if (!ok)
+                    break;
+                tc_fence_after();
+#pragma unroll
+                for (int g = 0; g < S::G; g++, kb++) {
+                    const int tap = kb / CB, c = kb % CB, dy = tap / 3;
+                    const uint64_t ad = sw128_desc(sw + (b * CB + c) * S::A_BLOCK + (dy * (C64_HW - 3) + tap) * ROW_BYTES,
+                                                   16, C64_HW * ROW_BYTES);
+                    const uint64_t bd = sw128_desc(sw + S::OFF_B + (s * S::G + g) * S::B_BLOCK, 16, 1024);
+#pragma unroll
+                    for (int k = 0; k < KB / 16; k++)
+                        umma_bf16(dt, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0);
+                }
+                umma_commit(&b_empty[s]);
+                if (++s == S::B_STAGES) {
+                    s = 0;
+                    phase ^= 1;
+                }
+            }
+            if (ok) {
+                umma_commit(&a_empty[b]);
+                umma_commit(&acc_full[acc]);
+            }
+        }
+        if (!ok) {
+            atomicOr(a.status, ST_TIMEOUT_MMA);
+            *abort_flag = 1;
+        }
+    } else if (warp >= 2 && warp < 6) {
+        const int q = warp & 3;
+        int it = 0;
+        for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x, it++) {
+            const int acc = it & 1;
+            int w0, h0, img;
+            place(tile, w0, h0, img);
+            // staged output, 64 channels of this warp's 32 pixels (8 x 4): buffer (it * BN / 64 + hf) & 1
+            auto stage = [&](int hf) {
+                return smem + S::OFF_OUT + ((it * (BN / 64) + hf) & 1) * S::HALF_BYTES + q * 32 * ROW_BYTES;
+            };
+            if (SLOPE && lane == 0) {
+                // the slopes into the staging buffers, once the stores have read them
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+#pragma unroll
+                for (int hf = 0; hf < BN / 64; hf++) {
+                    uint64_t *bar = &sl_full[2 * q + ((it * (BN / 64) + hf) & 1)];
+                    mbar_expect_tx(bar, 32 * ROW_BYTES);
+                    tma_load_4d(stage(hf), &map_slope, bar, n0 + 64 * hf, w0, h0 + 4 * q, img);
+                }
+            }
+            // the tensor-memory loads are warp-collective: take the decision per warp
+            bool ok = mbar_wait(&acc_full[acc], (it >> 1) & 1, a.status);
+#pragma unroll
+            for (int hf = 0; hf < BN / 64; hf++)
+                if (SLOPE) {
+                    const int u = it * (BN / 64) + hf;  // use of the buffer u & 1
+                    ok = ok && mbar_wait(&sl_full[2 * q + (u & 1)], (u >> 1) & 1, a.status);
+                }
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0)
+                    atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                break;
+            }
+            tc_fence_after();
+            const uint32_t td = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * BN);
+#pragma unroll 1
+            for (int hf = 0; hf < BN / 64; hf++) {
+                uint8_t *row = stage(hf) + lane * ROW_BYTES;
+                if (!SLOPE) {
+                    if (lane == 0)
+                        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(td + (uint32_t)(64 * hf + c0), v);
+                    if (has_bias) {
+#pragma unroll
+                        for (int i = 0; i < 32; i++) {
+                            const float z = v[i] + sbias[64 * hf + c0 + i];
+                            v[i] = a.epi == EPI_BIAS_LRELU ? lrelu(z) : z;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        uint4 *at = (uint4 *)(row + ((c0 / 8 + j) ^ (lane & 7)) * 16);
+                        if (SLOPE) {
+                            const uint4 u = *at;
+                            const bf16 *yb = (const bf16 *)&u;
+#pragma unroll
+                            for (int e = 0; e < 8; e++)
+                                v[8 * j + e] *= lrelu_slope(__bfloat162float(yb[e]));
+                        }
+                        uint4 u;
+                        __nv_bfloat162 *p2 = (__nv_bfloat162 *)&u;
+#pragma unroll
+                        for (int e = 0; e < 4; e++)
+                            p2[e] = __floats2bfloat162_rn(v[8 * j + 2 * e], v[8 * j + 2 * e + 1]);
+                        *at = u;
+                    }
+                }
+                fence_proxy_async_smem();
+                if (hf == BN / 64 - 1)
+                    tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (hf == BN / 64 - 1)
+                        mbar_arrive(&acc_empty[acc]);
+                    if (h0 + 4 * q < a.h)
+                        tma_store_4d(&map_out, stage(hf), n0 + 64 * hf, w0, h0 + 4 * q, img);
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+            }
+        }
+        if (lane == 0)
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, S::TMEM_COLS);
+    }
+}
+
+// --------------------------------------------------------------------------
 // Weight gradient of one tap: D[o][i] = sum_p dz[p][o] x[p + s_tap][i] over a
 // range of 64-pixel K blocks.  Both operands are loaded from the NHWC tensors
 // as they are, so they are MN-major (the 64 channels of one pixel form one

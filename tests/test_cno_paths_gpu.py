@@ -119,3 +119,21 @@ def test_64_channel_weight_gradients(n, h, w, cout):
     assert bool(((dw.double() - ref(dz, x)).abs() <= 2.0 ** -13 * ref(dz.abs(), x.abs()) + 1e-30).all())
     s = dz.double().sum((0, 1, 2))
     assert bool(((db.double() - s).abs() <= 2.0 ** -13 * dz.double().abs().sum((0, 1, 2)) + 1e-30).all())
+
+
+# streamed weights: one, two and four 64-channel blocks in, one, two and four out; whole, ragged and single tiles, several per block
+@pytest.mark.parametrize("cin,cout", [(64, 128), (64, 256), (128, 64), (128, 128), (128, 192), (128, 256), (256, 64), (256, 128), (256, 256)])
+@pytest.mark.parametrize("n,h,w", [(1, 1, 8), (2, 17, 16), (1, 33, 130), (3, 64, 128)])
+def test_wide_layers(n, h, w, cin, cout):
+    from paper_2511_09422_gb300 import cno
+    x, w32, b = _conv_case(n, h, w, cin, cout, h + w + cin)
+    wf, _ = cno.weights_to_bf16(w32)
+    ref, mag = _ref(x, wf, b)
+    for act in (True, False):
+        want = torch.where(ref > 0, ref, ref / 16) if act else ref
+        _inside(cno.conv3x3_forward(x, wf, b, act), want, mag, "forward")
+    ref, mag = _ref(x, wf)  # the weights read as Wd: a data gradient from cin to cout channels
+    _inside(cno.conv3x3_dgrad(x, wf), ref, mag, "dgrad")
+    slope = torch.randn((n, h, w, cout), device="cuda").to(torch.bfloat16)
+    k = torch.where(slope > 0, 1.0, 1.0 / 16).double()
+    _inside(cno.conv3x3_dgrad(x, wf, slope), ref * k, mag * k, "dgrad with slope")
