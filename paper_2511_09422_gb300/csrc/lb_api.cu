@@ -157,11 +157,13 @@ static std::string check_params(const lb_grid *g, const lb_params *p)
 // step time when it cuts the work into items(h) items.  An item runs h + 3 rows
 // one after another (its own, and the fill of the rings).  The warps of the wave
 // take the items in rounds of W; a row takes longer the more warps share a
-// scheduler (1.45 us with one, 2.1 us with two FP32 warps), and with many rounds
-// the last one is only partly filled.  Measured for heights 1 .. 16 (us per step):
+// scheduler (1.45 us with one, 2.1 us with two FP32 warps; 1.6, 2.5 and 2.8 us with one, two
+// and three of a half form), and with many rounds the last one is only partly
+// filled.  Measured for heights 1 .. 16 (us per step):
 //   film 64 x 256: 9.2 at 2 rows, 17.0 at 8;   512 x 256: 15.1 at 4, 23.5 at 8;
 //   256^2: 11.4 at 2, 17.5 at 8;   512^2: 25.5 at 8, 28.5 at 4, 32.2 at 3;
-//   1037 x 771 (D2Q5): 61.6 at 12, 64.0 at 8, 72.2 at 10;   1024^2: 87.8 at 10, 95.1 at 12.
+//   1037 x 771 (D2Q5): 61.6 at 12, 64.0 at 8, 72.2 at 10;   1024^2: 87.8 at 10, 95.1 at 12;
+//   F16: 512^2 26.6 at 6, 33.1 at 8, 29.9 at 3;   1024^2 76.7 at 16, 79.6 at 10, 87.1 at 8.
 // The estimate picks the best or the second best height in each of them.
 template <class Items>
 static int best_segment_rows(int kind, int max_rows, Items items)
@@ -169,13 +171,15 @@ static int best_segment_rows(int kind, int max_rows, Items items)
     const long long W = with_storage(kind, [](auto ps) {
         return 152LL * lbk::step_min_blocks<decltype(ps)>() * lbk::step_warps<decltype(ps)>();
     });
+    const bool half = kind == 1 || kind == 3;
     int best = 1;
     double least = 0.0;
     for (int h = 1; h <= max_rows; h++) {
         const long long n = items(h);
         const double waves = (double)n / (double)W, rounds = waves <= 8.0 ? std::ceil(waves) : waves + 0.5;
         const long long per_scheduler = ((n < W ? n : W) + 607) / 608;
-        const double cost = rounds * (h + 3) * (1.0 + 0.45 * (double)(per_scheduler - 1));
+        const double share = per_scheduler <= 1 ? 1.0 : (!half ? 1.45 : (per_scheduler == 2 ? 1.55 : 1.75));
+        const double cost = rounds * (h + 3) * share;
         if (h == 1 || cost < least) {
             least = cost;
             best = h;

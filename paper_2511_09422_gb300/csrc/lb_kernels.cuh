@@ -1035,7 +1035,7 @@ __host__ __device__ constexpr int win_elems()
     return win_bytes<PS>(S) / PS::esize(S);
 }
 
-// The rings of one warp under storage PS (windows of half sets take 96 bytes,
+// The rings of one warp under storage PS (windows of half sets take 80 bytes,
 // so a warp's rings are smaller and more warps fit on an SM).  PB = false:
 // the rings of a sweep that runs phase A alone (the diagnostics), without the
 // phase-A outputs, the staged (p, S) and the g pulls that only phase B reads
