@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
             const int th = t % a.tiles_h;
             const int img = t / a.tiles_h;
             const int w0 = tw * a.wt, h0 = th * a.ht;
+            int cb = 0, dx = -1, dy = -1;  // channel block and tap of kb
             for (int kb = 0; kb < a.kblocks; kb++, kc++) {
                 const int s = kc % S::STAGES;
                 const uint32_t use = kc / S::STAGES;
@@ -340,12 +341,17 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
                     *abort_flag = 1;
                     break;
                 }
-                const int tap = kb / a.cblocks, cb = kb - tap * a.cblocks;
-                const int dy = tap / 3 - 1, dx = tap % 3 - 1;
                 uint8_t *sa = smem + s * S::STAGE;
                 mbar_expect_tx(&full[s], S::STAGE);
                 tma_load_4d(sa, &map_x, &full[s], cb * KB, w0 + dx, h0 + dy, img);
                 tma_load_2d(sa + S::A_BYTES, &map_w, &full[s], kb * KB, n0);
+                if (++cb == a.cblocks) {
+                    cb = 0;
+                    if (++dx == 2) {
+                        dx = -1;
+                        dy++;
+                    }
+                }
             }
         }
     } else if (warp == 1 && lane == 0) {
@@ -1140,6 +1146,8 @@ __global__ void __launch_bounds__(192, 1)
 
     if (warp == 0 && lane == 0) {
         const uint32_t bytes = (two_m ? 2 : 1) * SUB_BYTES + S::B_BYTES;
+        // the K block's place, kept instead of divided for
+        int tw = kb_lo % a.tiles_w, th = kb_lo / a.tiles_w % a.tiles_h, img = kb_lo / a.tiles_w / a.tiles_h;
         for (int j = 0; j < nk && !*abort_flag; j++) {
             const int s = j % S::STAGES, it = j / S::STAGES;
             if (j >= S::STAGES && !mbar_wait(&empty[s], (it - 1) & 1, a.status)) {
@@ -1147,11 +1155,6 @@ __global__ void __launch_bounds__(192, 1)
                 *abort_flag = 1;
                 break;
             }
-            int kb = kb_lo + j;
-            const int tw = kb % a.tiles_w;
-            kb /= a.tiles_w;
-            const int th = kb % a.tiles_h;
-            const int img = kb / a.tiles_h;
             const int pw = tw * a.wt, ph = th * a.ht;
             uint8_t *st = smem + s * S::STAGE;
             mbar_expect_tx(&full[s], bytes);
@@ -1161,6 +1164,13 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
             for (int q = 0; q < BN / 64; q++)
                 tma_load_4d(st + S::A_BYTES + q * SUB_BYTES, &map_x, &full[s], n0 + 64 * q, pw + dx, ph + dy, img);
+            if (++tw == a.tiles_w) {
+                tw = 0;
+                if (++th == a.tiles_h) {
+                    th = 0;
+                    img++;
+                }
+            }
         }
     } else if (warp == 1 && lane == 0) {
         constexpr uint32_t idesc = idesc_bf16(BM, BN, 1, 1);
