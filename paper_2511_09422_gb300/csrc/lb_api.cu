@@ -359,10 +359,29 @@ static cudaError_t launch_step(const lbk::StepRec *rec, int ninst, long long nit
     });
 }
 
+// Constants of a read-out sweep (fields, diagnostics): the step's segments, except
+// that FP32 lattices of more than `waves` waves of them take `rows` rows.  A taller
+// segment fills the rings less often; with few waves it leaves the last one empty
+// (1024^2, fields 61 us at 10 rows, 67 at 32).  Step's own 12 rows / 24 / 32 rows, us:
+//   fields       2048^2 194/188/187, 3000 x 1500 206/199/201, 2500^2 282/268/273,
+//                3000^2 397/374/372, 4096^2 733/684/674;
+//   diagnostics  2048^2 153/154/154, 3000 x 1500 159/159/162, 2500^2 204/203/203,
+//                3000^2 277/268/271, 4096^2 487/468/473.
+// So the fields take 32 rows above 8 waves, and the diagnostics 24 above 16 (2500^2
+// has 14.5, 3000^2 has 20.8).
+static Consts read_consts(const lb_handle *h, int rows, int waves)
+{
+    Consts K = h->K;
+    const long long W = 152LL * lbk::step_min_blocks<lbk::PopF32>() * lbk::step_warps<lbk::PopF32>();
+    const long long items = (long long)((K.nx + LB_TX - 1) / LB_TX) * lbk::strip_segments(K.ny, K.segh);
+    if (h->kind == 0 && items > waves * W && rows > K.segh) K.segh = rows;
+    return K;
+}
+
 // The diagnostics sums and, in out[NRED], the status word (0: no non-finite value).
 static lb_status launch_reduce(lb_handle *h, double out[lbk::NRED + 1])
 {
-    const Consts &K = h->K;
+    const Consts K = read_consts(h, 24, 16);
     lbk::Buffers B = {};
     B.pin = h->pops[h->cur];
     B.ain = h->aux[h->cur];
@@ -619,7 +638,7 @@ extern "C" lb_status lb_get_fields(lb_handle *h, float *phi, float *T, float *fs
 {
     if (!h) return LB_ERR_INVALID_ARG;
     if (h->sticky != LB_OK) return h->sticky;
-    const Consts &K = h->K;
+    const Consts K = read_consts(h, 32, 8);
     // outputs in this device's memory are written in place, others by way of the 7-plane field buffer (dense)
     float *dst[7] = {phi, T, fs, C, ux, uy, p};
     const size_t n = (size_t)K.nx * K.ny;

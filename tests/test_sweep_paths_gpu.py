@@ -66,6 +66,23 @@ def test_segment_heights_do_not_change_the_step(ny):
         assert np.array_equal(a[n], got[n]), n
 
 
+# a lattice repeated in x: above 8 waves the fields, above 16 also the diagnostics are read in taller
+# segments than the narrow lattice's, the last of them not whole; half storage keeps the step's
+@pytest.mark.parametrize("ny", [1001, 1711])
+@pytest.mark.parametrize("storage", [(0, 0), (1, 0), (2, 0), (0, 1)], ids=["f32", "f16", "f16h32", "d2q5"])
+def test_repeated_lattice_reads_out_repeated_fields(ny, storage):
+    w = W.parity_droplet(nx=512, ny=ny, steps=2)
+    f = {k: np.asarray(v, np.float32) for k, v in w["fields"].items()}
+    a, ra = _run(w, f, storage, 2)
+    big = W.parity_droplet(nx=4096, ny=ny, steps=2)
+    big["params"] = w["params"]
+    b, rb = _run(big, {n: np.tile(v, (1, 8)) for n, v in f.items()}, storage, 2)
+    for n in FIELDS:
+        assert np.array_equal(np.tile(a[n], (1, 8)), b[n]), n
+    # compensated sums over other segments, terms of both signs: 1e-12 of the sum and of one a cell
+    assert np.allclose(8 * ra[:5], rb[:5], rtol=1e-12, atol=1e-12 * 4096 * ny)
+
+
 @pytest.mark.parametrize("nx,ny", [(5, 4), (30, 7), (64, 33), (101, 40)])
 def test_device_read_out_matches_host(nx, ny):
     w = W.parity_droplet(nx=nx, ny=ny, steps=3)
