@@ -1213,8 +1213,8 @@ __device__ __noinline__ void check_wide(double (&wide)[6], double f, double fe, 
 }
 
 constexpr int CHK_THREADS = 256;
-__global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *__restrict__ phi, const float *__restrict__ fs,
-                                                                 const float *__restrict__ T, HCoef hc, int nx, int ny,
+__global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *phi, const float *fs,
+                                                                 const float *T, HCoef hc, int nx, int ny,
                                                                  double *__restrict__ part)
 {
     cnok::grid_begin();
@@ -1315,7 +1315,7 @@ __global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *__
 }
 
 // The blocks' sums in a fixed order: thread (k, j) takes blocks j, j + 32, ...
-__global__ void __launch_bounds__(32 * NCHK) field_total_kernel(const double *__restrict__ part, int blocks,
+__global__ void __launch_bounds__(32 * NCHK) field_total_kernel(const double *part, int blocks,
                                                                 double *__restrict__ out)
 {
     cnok::grid_begin();

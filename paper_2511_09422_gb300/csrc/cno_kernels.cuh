@@ -35,7 +35,10 @@ constexpr unsigned ST_TIMEOUT_PRODUCER = 1u, ST_TIMEOUT_MMA = 2u, ST_TIMEOUT_EPI
 // kernel in front of it has ended.  grid_begin waits for that kernel's end (its
 // writes are then visible) and only then lets the kernel behind this one start its
 // blocks, so at most two are ever in flight.  Every kernel launched that way calls
-// it before its first access to global memory.
+// it before its first access to global memory.  Its inputs may be written while it
+// is resident, so it must not read them as read-only data: no __ldg, and no
+// "const T *__restrict__" input, which lets the compiler choose such a load and move
+// it over the wait (__restrict__ on what it writes is enough to overlap its loads).
 __device__ __forceinline__ void grid_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -433,7 +436,7 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
                     const uint4 *ys = (const uint4 *)(a.slope_src + pix * a.cout + oc);
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        uint4 u = __ldg(&ys[j]);
+                        uint4 u = ys[j];
                         const bf16 *yb = (const bf16 *)&u;
 #pragma unroll
                         for (int e = 0; e < 8; e++)
@@ -1429,7 +1432,7 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8])
 }
 
 // dW[i] = sum over splits s (in order) of partial[s][i]; eight reads in flight
-__global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restrict__ partial, int splits,
+__global__ void __launch_bounds__(256) sum_partials_kernel(const float *partial, int splits,
                                                            long long count, float *__restrict__ out)
 {
     grid_begin();
@@ -1458,7 +1461,7 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restri
 // warp's loads are contiguous; the threads of one channel group are then added
 // in shared memory in a fixed order.  Bound by the read of dz: each thread keeps
 // eight loads in flight (with one, 50 us for 134 MB, 2.7 TB/s).
-__global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *__restrict__ dz, long long npix, int c,
+__global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *dz, long long npix, int c,
                                                           long long ppb, float *__restrict__ partial)
 {
     grid_begin();
@@ -1507,7 +1510,7 @@ __global__ void __launch_bounds__(256) channel_sum_kernel(const bf16 *__restrict
 
 // Bias gradient, second pass: db[ch] = sum of partial[b][ch] over the blocks, one
 // block of 32 channels x 32 block groups, added in a fixed order.
-__global__ void __launch_bounds__(1024) channel_total_kernel(const float *__restrict__ partial, int blocks, int c,
+__global__ void __launch_bounds__(1024) channel_total_kernel(const float *partial, int blocks, int c,
                                                              float *__restrict__ db)
 {
     grid_begin();
@@ -1531,7 +1534,7 @@ __global__ void __launch_bounds__(1024) channel_total_kernel(const float *__rest
 // Elementwise kernels on NHWC bf16 tensors, 8 channels (16 bytes) per thread.
 // --------------------------------------------------------------------------
 // y[n][h][w] = mean of x[n][2h..2h+1][2w..2w+1]; x is n x 2ho x 2wo
-__global__ void pool2_kernel(const bf16 *__restrict__ x, int n, int ho, int wo, int c, bf16 *__restrict__ y)
+__global__ void pool2_kernel(const bf16 *x, int n, int ho, int wo, int c, bf16 *__restrict__ y)
 {
     grid_begin();
     const int cv = c / 8;
@@ -1565,7 +1568,7 @@ __global__ void pool2_kernel(const bf16 *__restrict__ x, int n, int ho, int wo, 
 }
 
 // u = up2(x) + skip; x is n x h/2 x w/2, skip and u n x h x w
-__global__ void up_add_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ skip, int n, int h, int w, int c,
+__global__ void up_add_kernel(const bf16 *x, const bf16 *skip, int n, int h, int w, int c,
                               bf16 *__restrict__ u)
 {
     grid_begin();
@@ -1592,7 +1595,7 @@ __global__ void up_add_kernel(const bf16 *__restrict__ x, const bf16 *__restrict
 
 // Backward of u = up2(x) + skip followed by x = lrelu(.): dz[p] = slope(y[p]) *
 // sum of du over the 2x2 block of p (y = x, the coarse activation)
-__global__ void up_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restrict__ y, int n, int ho, int wo, int c,
+__global__ void up_bwd_kernel(const bf16 *du, const bf16 *y, int n, int ho, int wo, int c,
                               bf16 *__restrict__ dz)
 {
     grid_begin();
@@ -1631,7 +1634,7 @@ __global__ void up_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restric
 // Backward at an encoder output e that feeds both a skip addition (gradient
 // du) and pooling (gradient dp, at half resolution), followed by e = lrelu(.):
 // dz[p] = slope(e[p]) * (du[p] + dp[p / 2] / 4)
-__global__ void pool_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restrict__ dp, const bf16 *__restrict__ e,
+__global__ void pool_bwd_kernel(const bf16 *du, const bf16 *dp, const bf16 *e,
                                 int n, int h, int w, int c, bf16 *__restrict__ dz)
 {
     grid_begin();
@@ -1665,7 +1668,7 @@ __global__ void pool_bwd_kernel(const bf16 *__restrict__ du, const bf16 *__restr
 // contiguous bytes per store.  The squares are summed as exact FP32 pairs with
 // compensation.  Bound by the write of dout; in FP64, one row per thread, this
 // took 259 us for 16 x 256^2 (134 MB).
-__global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ out, const float *__restrict__ target,
+__global__ void __launch_bounds__(256) mse_kernel(const float *out, const float *target,
                                                   int nf, long long npix, int c, double inv_count,
                                                   bf16 *__restrict__ dout, double *__restrict__ partial)
 {
@@ -1731,7 +1734,7 @@ __global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ out,
 // Adam (Kingma and Ba, Algorithm 1) on FP32 master parameters; omb1 = 1 - beta1,
 // omb2 = 1 - beta2, c1 = 1 - beta1^t, c2 = 1 - beta2^t, all rounded from FP64 on
 // the host so that omb1 / c1 = omb2 / c2 = 1 exactly at t = 1.
-__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
+__global__ void adam_kernel(float *__restrict__ p, const float *g, float *__restrict__ m,
                             float *__restrict__ v, long long count, float lr, float beta1, float beta2, float omb1,
                             float omb2, float eps, float c1, float c2)
 {
@@ -1767,7 +1770,7 @@ __global__ void __launch_bounds__(256) weights_to_bf16_kernel(const __grid_const
     while (l + 1 < a.n && (int)blockIdx.x >= a.block0[l + 1])
         l++;
     const int cout = a.cout[l], cin = a.cin[l];
-    const float *__restrict__ w = a.w[l];
+    const float *w = a.w[l];
     bf16 *__restrict__ wf = a.wf[l], *__restrict__ wd = a.wd[l];
     const long long total = (long long)cout * 9 * cin, step = (long long)(a.block0[l + 1] - a.block0[l]) * blockDim.x;
     for (long long idx = (blockIdx.x - a.block0[l]) * (long long)blockDim.x + threadIdx.x; idx < total; idx += step) {
