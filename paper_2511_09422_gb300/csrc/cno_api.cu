@@ -1155,61 +1155,56 @@ __global__ void __launch_bounds__(256) apply_update_kernel(FieldPtrs src, FieldO
 }
 
 // Sums of phi, chi, f_s, 1 - phi^2, |grad phi|, the minimum and maximum of T, and
-// the sum of rho H.  FP64 is the scarce pipe of this GPU (2 lane operations per
-// cycle and SM), and evaluating and adding a cell's terms in FP64 took 114 us at
-// 1024^2.  Each term is formed as an unevaluated FP32 pair from error-free sums and
-// products (relative error of order 2^-44) and added with compensation, so that the
-// sums keep FP64 accuracy; only one conversion per warp and sum is left.  A cell with
-// a value beyond DIRECT (infinities and NaN among them), where the products could
-// overflow FP32, is evaluated and added in FP64.
+// the sum of rho H.  Evaluating and adding a cell's terms in FP64 took 114 us at
+// 1024^2.  Here they are formed and added as FP32 expansions (f3, in cno_kernels.cuh)
+// that keep more than FP64's bits, and FP64 is left for the sums of the blocks'
+// warps.  Where an operand or product is so large (DIRECT, infinities and NaN) or so
+// small (the gradient below 2^-40, rho H below 2^-80) that an FP32 product or its rounding
+// error would leave the range, the cell's term is evaluated and added in FP64.
 constexpr int NCHK = 8;
 constexpr float DIRECT = 1e12f;
+constexpr float GRAD2_MIN = 8.2718061e-25f, CAP_MIN = 8.6736174e-19f, HEAT_MIN = 8.2718061e-25f;  // 2^-80, 2^-60, 2^-80
+constexpr float LATENT_MIN = 9.0949470e-13f;                                                        // 2^-40
 struct HCoef {
     float cl, cs, cg, lat;
-    int on, wide;  // wide: a coefficient beyond DIRECT
+    int on, wide;  // wide: a coefficient out of range
 };
-struct ff {
-    float h, l;  // h + l, |l| small beside h
-};
-__device__ __forceinline__ ff ff_sum(float a, float b)  // exact
-{
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ ff ff_add(ff a, ff b)
-{
-    const ff s = ff_sum(a.h, b.h);
-    return ff_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ ff ff_mul(ff a, ff b)
-{
-    const float p = __fmul_rn(a.h, b.h);
-    return {p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.h, -a.l}; }
 
-__device__ __forceinline__ void check_add(ff &a, ff x)
+// A cell in FP64, the terms of the bits `which` added to the sums `wide`: f its phi,
+// fe, fw, fn, fso the neighbours (gradient scale gys in y).
+constexpr unsigned TERM_GRAD = 1u << 4, TERM_HEAT = 1u << 5, ALL_TERMS = 63u;
+__device__ __noinline__ void check_wide(double (&wide)[6], unsigned which, double f, double fe, double fw, double fn,
+                                        double fso, double gys, double fs, double t, const HCoef &hc)
 {
-    const ff t = ff_sum(a.h, x.h);
-    a = {t.h, __fadd_rn(a.l, __fadd_rn(t.l, x.l))};
-}
-
-// A cell in FP64, added to the sums `wide`: f its phi, fe, fw, fn, fso the neighbours
-// (gradient scale gys in y).
-__device__ __noinline__ void check_wide(double (&wide)[6], double f, double fe, double fw, double fn, double fso, double gys,
-                                        double fs, double t, const HCoef &hc)
-{
-    const double gx = 0.5 * (fe - fw), gy = gys * (fn - fso);
     const double chi = fmin(fmax(0.5 * (1.0 + f), 0.0), 1.0);
-    wide[0] += f;
-    wide[1] += chi;
-    wide[2] += fs;
-    wide[3] += 1.0 - f * f;
-    wide[4] += sqrt(gx * gx + gy * gy);
-    if (hc.on) {
+    if (which == ALL_TERMS) {
+        wide[0] += f;
+        wide[1] += chi;
+        wide[2] += fs;
+        wide[3] += 1.0 - f * f;
+    }
+    if (which & TERM_GRAD) {
+        const double gx = 0.5 * (fe - fw), gy = gys * (fn - fso);
+        wide[4] += sqrt(gx * gx + gy * gy);
+    }
+    if ((which & TERM_HEAT) && hc.on) {
         const double sol = fmin(fmax(fs, 0.0), chi);
         wide[5] += t * (sol * hc.cs + (chi - sol) * hc.cl + (1.0 - chi) * hc.cg) + (double)hc.lat * (chi - sol);
     }
+}
+
+// sum += sqrt(q): the FP32 root and two Newton corrections of it
+__device__ __forceinline__ void add_root(cnok::f3 &sum, const cnok::f3 &q)
+{
+    using namespace cnok;
+    const float r = __fsqrt_rn(q.h), inv = __fdiv_rn(0.5f, r);
+    const f2 p = two_prod(r, r);
+    // q - r^2 = t + lo (the difference of the heads is exact), then q - (r + c)^2
+    const f2 a = two_sum(__fsub_rn(q.h, p.s), -p.e), t = two_sum(a.s, q.m);
+    const float lo = __fadd_rn(__fadd_rn(a.e, t.e), q.l), c = __fmul_rn(t.s, inv);
+    const f2 b = two_prod(2.0f * r, c);
+    const float rest = __fadd_rn(__fmaf_rn(-c, c, __fsub_rn(__fsub_rn(t.s, b.s), b.e)), lo);
+    f3_add(sum, r, c, __fmul_rn(rest, inv));
 }
 
 constexpr int CHK_THREADS = 256;
@@ -1217,15 +1212,11 @@ __global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *ph
                                                                  const float *T, HCoef hc, int nx, int ny,
                                                                  double *__restrict__ part)
 {
-    cnok::grid_begin();
-    ff sum[6];       // phi, chi, f_s, 1 - phi^2, |grad phi|, rho H
-    double wide[6];  // the cells evaluated in FP64
-    float lo = INFINITY, hi = -INFINITY;  // T
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        sum[k] = {0.0f, 0.0f};
-        wide[k] = 0.0;
-    }
+    using namespace cnok;
+    grid_begin();
+    f3 sum[6] = {};                        // phi, chi, f_s, 1 - phi^2, |grad phi|, rho H
+    double wide[6] = {0, 0, 0, 0, 0, 0};   // the terms taken in FP64
+    float lo = INFINITY, hi = -INFINITY;   // T
     for (int y = blockIdx.x; y < ny; y += gridDim.x) {
         const float *row = phi + (long long)y * nx;
         // rows of the central difference in y, one-sided next to the walls
@@ -1241,76 +1232,108 @@ __global__ void __launch_bounds__(CHK_THREADS) field_sums_kernel(const float *ph
             const float nb = fmaxf(fmaxf(fabsf(fe), fabsf(fw)), fmaxf(fabsf(fn), fabsf(fso)));
             const float all = fabsf(f) + fabsf(sol) + fabsf(t) + fabsf(fe) + fabsf(fw) + fabsf(fn) + fabsf(fso);  // NaN kept
             if (hc.wide || !(fmaxf(mag, nb) < DIRECT) || !(all < INFINITY)) {
-                check_wide(wide, f, fe, fw, fn, fso, gys, sol, t, hc);
+                check_wide(wide, ALL_TERMS, f, fe, fw, fn, fso, gys, sol, t, hc);
                 continue;
             }
-            check_add(sum[0], {f, 0.0f});
-            // chi = clamp((1 + phi) / 2)
-            ff chi = ff_sum(1.0f, f);
-            chi = {0.5f * chi.h, 0.5f * chi.l};
-            if (!(f > -1.0f)) chi = {0.0f, 0.0f};
-            if (!(f < 1.0f)) chi = {1.0f, 0.0f};
-            check_add(sum[1], chi);
-            check_add(sum[2], {sol, 0.0f});
-            const ff ff0 = {f, 0.0f};
-            check_add(sum[3], ff_add({1.0f, 0.0f}, ff_neg(ff_mul(ff0, ff0))));
-            // |grad phi| = sqrt(gx^2 + gy^2): FP32 root and one Newton correction
-            ff gx = ff_sum(fe, -fw), gy = ff_sum(fn, -fso);
-            gx = {0.5f * gx.h, 0.5f * gx.l};
-            gy = {gys * gy.h, gys * gy.l};
-            const ff q = ff_add(ff_mul(gx, gx), ff_mul(gy, gy));
-            const float r = sqrtf(q.h);
-            if (r > 0.0f) {
-                const float res = __fadd_rn(__fmaf_rn(-r, r, q.h), q.l);
-                check_add(sum[4], {r, __fdiv_rn(res, 2.0f * r)});
+            f3_add(sum[0], f);
+            // chi = clamp((1 + phi) / 2) and 1 - chi, both exact
+            f2 chi = two_sum(1.0f, f), gas = two_sum(1.0f, -f);
+            chi = {0.5f * chi.s, 0.5f * chi.e};
+            gas = {0.5f * gas.s, 0.5f * gas.e};
+            if (!(f > -1.0f)) chi = {0.0f, 0.0f}, gas = {1.0f, 0.0f};
+            if (!(f < 1.0f)) chi = {1.0f, 0.0f}, gas = {0.0f, 0.0f};
+            f3_add(sum[1], chi.s, chi.e);
+            f3_add(sum[2], sol);
+            {
+                const f2 p = two_prod(f, f), a = two_sum(1.0f, -p.s), b = two_sum(a.e, -p.e);
+                f3_add(sum[3], a.s, b.s, b.e);
             }
+            unsigned small = 0u;
+            // |grad phi| = sqrt(gx^2 + gy^2), the differences exact
+            f2 gx = two_sum(fe, -fw), gy = two_sum(fn, -fso);
+            gx = {0.5f * gx.s, 0.5f * gx.e};
+            gy = {gys * gy.s, gys * gy.e};
+            f3 q = {0.0f, 0.0f, 0.0f};
+            f3_add_product(q, gx.s, gx.s);
+            f3_add_product(q, gy.s, gy.s);
+            f3_add_product(q, 2.0f * gx.s, gx.e);
+            f3_add_product(q, 2.0f * gy.s, gy.e);
+            q.l = __fadd_rn(q.l, __fmaf_rn(gx.e, gx.e, __fmul_rn(gy.e, gy.e)));
+            if (q.h >= GRAD2_MIN)
+                add_root(sum[4], q);
+            else if (gx.s != 0.0f || gy.s != 0.0f)
+                small = TERM_GRAD;
             if (hc.on) {
-                // sol = clamp(f_s, 0, chi); rho H = T (sol c_s + d c_l + (1 - chi) c_g) + lat d, d = chi - sol
-                ff so = {fmaxf(sol, 0.0f), 0.0f};
-                if (so.h > chi.h || (so.h == chi.h && chi.l < 0.0f)) so = chi;
-                const ff d = ff_add(chi, ff_neg(so)), gas = ff_add({1.0f, 0.0f}, ff_neg(chi));
-                const ff cap = ff_add(ff_add(ff_mul(so, {hc.cs, 0.0f}), ff_mul(d, {hc.cl, 0.0f})), ff_mul(gas, {hc.cg, 0.0f}));
-                check_add(sum[5], ff_add(ff_mul({t, 0.0f}, cap), ff_mul(d, {hc.lat, 0.0f})));
+                // so = clamp(f_s, 0, chi); rho H = T (so c_s + d c_l + (1 - chi) c_g) + lat d, d = chi - so
+                f2 so = {fmaxf(sol, 0.0f), 0.0f}, d = {0.0f, 0.0f};
+                float dl = 0.0f;  // d.s + d.e + dl, exact
+                if (so.s > chi.s || (so.s == chi.s && chi.e < 0.0f)) {
+                    so = chi;
+                } else {
+                    const f2 a = two_sum(chi.s, -so.s), b = two_sum(a.e, chi.e);
+                    d = two_sum(a.s, b.s);
+                    dl = b.e;
+                }
+                f3 cap = {0.0f, 0.0f, 0.0f};
+                f3_add_product(cap, so.s, hc.cs);
+                f3_add_product(cap, d.s, hc.cl);
+                f3_add_product(cap, gas.s, hc.cg);
+                f3_add_product(cap, so.e, hc.cs);
+                f3_add_product(cap, d.e, hc.cl);
+                f3_add_product(cap, gas.e, hc.cg);
+                cap.l = __fmaf_rn(dl, hc.cl, cap.l);
+                if (t == 0.0f || (cap.h >= CAP_MIN && fabsf(t) * cap.h >= HEAT_MIN)) {
+                    f3_add_product(sum[5], t, cap.h);
+                    f3_add_product(sum[5], t, cap.m);
+                    f3_add_product(sum[5], d.s, hc.lat);
+                    f3_add_product(sum[5], d.e, hc.lat);
+                    sum[5].l = __fadd_rn(sum[5].l, __fmaf_rn(t, cap.l, __fmul_rn(dl, hc.lat)));
+                } else {
+                    small |= TERM_HEAT;
+                }
             }
+            if (small)
+                check_wide(wide, small, f, fe, fw, fn, fso, gys, sol, t, hc);
         }
     }
-    // the warp's sums in a fixed order, still as pairs, then the block's in FP64
-    __shared__ double red[CHK_THREADS / 32][NCHK];
+    // the warps' sums in a fixed order, still as expansions, then the block's in FP64
+    __shared__ f3 red[CHK_THREADS / 32][6];
+    __shared__ double wred[CHK_THREADS / 32][6];
+    __shared__ float tred[CHK_THREADS / 32][2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    bool any_wide = false;
-#pragma unroll
-    for (int k = 0; k < 6; k++) any_wide = any_wide || wide[k] != 0.0;  // true for NaN too
-    any_wide = __any_sync(0xffffffffu, any_wide);
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-        ff v = sum[k];
-        for (int o = 16; o > 0; o >>= 1) {
-            const ff u = {__shfl_down_sync(0xffffffffu, v.h, o), __shfl_down_sync(0xffffffffu, v.l, o)};
-            check_add(v, u);
+        f3_warp_sum(sum[k]);
+        if (__any_sync(0xffffffffu, wide[k] != 0.0))  // true for NaN
+            for (int o = 16; o > 0; o >>= 1) wide[k] += __shfl_down_sync(0xffffffffu, wide[k], o);
+        if (lane == 0) {
+            red[w][k] = sum[k];
+            wred[w][k] = wide[k];
         }
-        double s = (double)v.h + (double)v.l;
-        if (any_wide) {
-            double wd = wide[k];
-            for (int o = 16; o > 0; o >>= 1) wd += __shfl_down_sync(0xffffffffu, wd, o);
-            s += wd;
-        }
-        if (lane == 0) red[w][k < 5 ? k : 7] = s;
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fminf(lo, __shfl_down_sync(0xffffffffu, lo, o));
         hi = fmaxf(hi, __shfl_down_sync(0xffffffffu, hi, o));
     }
     if (lane == 0) {
-        red[w][5] = lo;
-        red[w][6] = hi;
+        tred[w][0] = lo;
+        tred[w][1] = hi;
     }
     __syncthreads();
-    if (threadIdx.x < NCHK) {
+    if (threadIdx.x < 6) {
         const int k = threadIdx.x;
-        double s = red[0][k];
-        for (int j = 1; j < CHK_THREADS / 32; j++)
-            s = k == 5 ? fmin(s, red[j][k]) : (k == 6 ? fmax(s, red[j][k]) : s + red[j][k]);
-        part[(long long)blockIdx.x * NCHK + k] = s;
+        f3 v = red[0][k];
+        double s = wred[0][k];
+        for (int j = 1; j < CHK_THREADS / 32; j++) {
+            f3_add(v, red[j][k].h, red[j][k].m, red[j][k].l);
+            s += wred[j][k];
+        }
+        part[(long long)blockIdx.x * NCHK + (k < 5 ? k : 7)] = f3_value(v) + s;
+    } else if (threadIdx.x < 8) {
+        const int k = threadIdx.x - 6;
+        float v = tred[0][k];
+        for (int j = 1; j < CHK_THREADS / 32; j++) v = k == 0 ? fminf(v, tred[j][k]) : fmaxf(v, tred[j][k]);
+        part[(long long)blockIdx.x * NCHK + 5 + k] = v;
     }
 }
 
@@ -1467,6 +1490,8 @@ extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const 
         for (int k = 0; k < 4; k++)
             if (!(std::fabs(hcoef[k]) < DIRECT))
                 hc.wide = 1;
+        if (hc.lat != 0.0f && std::fabs(hc.lat) < LATENT_MIN)
+            hc.wide = 1;
     }
     CheckSlot slot;
     CS(check_slot_take(dev, &slot));

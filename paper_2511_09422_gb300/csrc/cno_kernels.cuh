@@ -1660,29 +1660,82 @@ __global__ void pool_bwd_kernel(const bf16 *du, const bf16 *dp, const bf16 *e,
     }
 }
 
+// --------------------------------------------------------------------------
+// Sums to FP64's accuracy from FP32 operations.  FP64 is the scarce pipe of this
+// GPU (2 lane operations a cycle and SM).  A sum is held as three floats, h + m + l;
+// sums and products of floats are exact as pairs (Knuth's TwoSum; an FMA for the
+// product), so what is added to it loses nothing down to about 2^-68 of the sum.
+// Products are exact as long as their rounding error does not underflow: the
+// callers send operands too small or too large for that to FP64.
+// --------------------------------------------------------------------------
+struct f2 {
+    float s, e;  // s + e: the result rounded, and its rounding error
+};
+struct f3 {
+    float h, m, l;
+};
+__device__ __forceinline__ f2 two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ f2 two_prod(float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+// a += x
+__device__ __forceinline__ void f3_add(f3 &a, float x)
+{
+    const f2 s = two_sum(a.h, x), t = two_sum(a.m, s.e), r = two_sum(s.s, t.s);
+    a.h = r.s;
+    a.m = r.e;
+    a.l = __fadd_rn(a.l, t.e);
+}
+// a += x + x1 + x2, each small beside the one before it
+__device__ __forceinline__ void f3_add(f3 &a, float x, float x1, float x2 = 0.0f)
+{
+    const f2 s = two_sum(a.h, x), t = two_sum(a.m, s.e), u = two_sum(t.s, x1), r = two_sum(s.s, u.s);
+    a.h = r.s;
+    a.m = r.e;
+    a.l = __fadd_rn(a.l, __fadd_rn(__fadd_rn(t.e, u.e), x2));
+}
+// a += x c
+__device__ __forceinline__ void f3_add_product(f3 &a, float x, float c)
+{
+    const f2 p = two_prod(x, c);
+    f3_add(a, p.s, p.e);
+}
+// The warp's sums in lane 0, in a fixed order.
+__device__ __forceinline__ void f3_warp_sum(f3 &a, int lanes = 32)
+{
+    for (int o = lanes / 2; o > 0; o >>= 1)
+        f3_add(a, __shfl_down_sync(0xffffffffu, a.h, o), __shfl_down_sync(0xffffffffu, a.m, o),
+               __shfl_down_sync(0xffffffffu, a.l, o));
+}
+__device__ __forceinline__ double f3_value(const f3 &a) { return (double)a.h + ((double)a.m + (double)a.l); }
+
 // Mean squared error over the first nf <= 8 channels of out (FP32, 8 per pixel)
 // against target (FP32, nf per pixel).  dout (bf16, c per pixel) gets 2 (out -
 // target) / count on those channels and 0 elsewhere; each block adds its squared
 // errors into partial[block] (FP64).  A warp takes 32 pixels: each lane forms the
 // gradient of its pixel, and the warp writes the pixels' rows in order, 512
-// contiguous bytes per store.  The squares are summed as exact FP32 pairs with
-// compensation.  Bound by the write of dout; in FP64, one row per thread, this
-// took 259 us for 16 x 256^2 (134 MB).
+// contiguous bytes per store.  The squares are exact pairs, added as above; a
+// difference beyond 2^-48 .. 1e12 (NaN too) is squared and added in FP64.  Bound by
+// the write of dout; in FP64, one row per thread, this took 259 us for 16 x 256^2
+// (134 MB).
+constexpr float SQUARE_MIN = 3.5527137e-15f, SQUARE_MAX = 1e12f;  // 2^-48
 __global__ void __launch_bounds__(256) mse_kernel(const float *out, const float *target,
                                                   int nf, long long npix, int c, double inv_count,
                                                   bf16 *__restrict__ dout, double *__restrict__ partial)
 {
     grid_begin();
-    __shared__ double red[8];
+    __shared__ f3 red[8];
+    __shared__ double wred[8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cv = c / 8;
     const float scale = (float)(2.0 * inv_count);
-    float hi = 0.0f, lo = 0.0f;  // sum of squares
-    double wide = 0.0;           // of differences beyond 1e12, NaN and infinities
-    auto add = [&](float x, float e) {  // hi + lo += x + e, the rounding error kept
-        const float s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb))));
-        hi = s;
-    };
+    f3 sum = {0.0f, 0.0f, 0.0f};
+    double wide = 0.0;  // squares taken in FP64
     for (long long g = blockIdx.x * 8LL + w; 32 * g < npix; g += gridDim.x * 8LL) {
         const long long p = 32 * g + lane;
         float d[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -1698,12 +1751,10 @@ __global__ void __launch_bounds__(256) mse_kernel(const float *out, const float 
 #pragma unroll
         for (int k = 0; k < 8; k++) {
             gr[k] = scale * d[k];
-            if (fabsf(d[k]) < 1e12f) {
-                const float sq = __fmul_rn(d[k], d[k]);
-                add(sq, __fmaf_rn(d[k], d[k], -sq));
-            } else {
+            if (fabsf(d[k]) >= SQUARE_MIN && fabsf(d[k]) < SQUARE_MAX)
+                f3_add_product(sum, d[k], d[k]);
+            else if (d[k] != 0.0f)
                 wide += (double)d[k] * (double)d[k];
-            }
         }
         const uint4 mine = pack8(gr);
         uint4 *row = (uint4 *)dout + 32 * g * cv;
@@ -1718,16 +1769,26 @@ __global__ void __launch_bounds__(256) mse_kernel(const float *out, const float 
                 row[q] = chunk == 0 ? u : make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    double s = (double)hi + (double)lo + wide;
-    for (int o = 16; o > 0; o >>= 1)
-        s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0)
-        red[w] = s;
+    // the warps, then the block, in a fixed order
+    f3_warp_sum(sum);
+    if (__any_sync(0xffffffffu, wide != 0.0))  // true for NaN
+        for (int o = 16; o > 0; o >>= 1)
+            wide += __shfl_down_sync(0xffffffffu, wide, o);
+    if (lane == 0) {
+        red[w] = sum;
+        wred[w] = wide;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int j = 1; j < 8; j++)
-            s += red[j];
-        partial[blockIdx.x] = s;
+    if (w == 0) {
+        f3 s = red[lane & 7];
+        f3_warp_sum(s, 8);
+        if (lane == 0) {
+            double t = f3_value(s);
+            for (int j = 0; j < 8; j++)
+                if (wred[j] != 0.0)
+                    t += wred[j];
+            partial[blockIdx.x] = t;
+        }
     }
 }
 
