@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "cno.h"
+#include "cno_dispatch.hpp"
 #include "cno_kernels.cuh"
 
 using cnok::bf16;
@@ -235,7 +236,8 @@ static cno_status launch_conv64(const void *in, const void *wmat, const void *sl
         CS(map_nhwc(&mo, a.out, a.n, a.h, a.w, a.cout, cnok::C64_W, 4));
     if (SLOPE)
         CS(map_nhwc(&ms, slope_src, a.n, a.h, a.w, a.cout, cnok::C64_W, cnok::C64_H));
-    const dim3 grid(std::min(a.tiles, num_sms()), BN == 64 ? a.cout / 64 : 1);
+    const int nblocks = BN == 64 ? a.cout / 64 : 1;
+    const dim3 grid(cnok::persistent_ctas(a.tiles, nblocks, num_sms()), nblocks);
     CK(launch(cnok::conv64_kernel<BN, SLOPE>, grid, 192, S::SMEM, st, mx, mw, mo, ms, a));
     return CNO_OK;
 }
@@ -259,7 +261,7 @@ static cno_status launch_conv_halo(const void *in, const void *wmat, const void 
     if (SLOPE)
         CS(map_nhwc(&ms, slope_src, a.n, a.h, a.w, a.cout, cnok::C64_W, 4));
     const int nblocks = a.cout / S::BN;
-    const dim3 grid(std::min(a.tiles, std::max(1, num_sms() / nblocks)), nblocks);
+    const dim3 grid(cnok::persistent_ctas(a.tiles, nblocks, num_sms()), nblocks);
     CK(launch(cnok::conv_halo_kernel<CB, SLOPE>, grid, 224, S::SMEM, st, mx, mw, mo, ms, a));
     return CNO_OK;
 }
