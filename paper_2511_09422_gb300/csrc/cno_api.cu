@@ -211,13 +211,6 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
     return CNO_OK;
 }
 
-// Which kernel takes a convolution: 64 -> 64, 192 channels (and the FP32 head) conv64_kernel,
-// 64 or 128 -> 128, 256 conv_halo_kernel, others conv_fprop_kernel, and all of
-// them where the tiles of 8 x 16 pixels are badly filled: HALO_TILES is the number
-// of them per tile of 128 pixels in a row up to which the first two are the faster ones
-// (at one row of pixels, sixteen to one, they compute mostly padding).
-constexpr double HALO_TILES = 1.4;
-
 template <int BN, bool SLOPE>
 static cno_status launch_conv64(const void *in, const void *wmat, const void *slope_src, const cnok::ConvArgs &a,
                                 cudaStream_t st)
@@ -322,31 +315,24 @@ static cno_status conv_launch(const void *in, int n, int h, int w, int cin, cons
     const long long tiles = (long long)n * a.tiles_w * a.tiles_h;
     if (tiles > 0x7fffffffLL)
         return fail(CNO_ERR_INVALID_ARG, "too many tiles");
-    const bool head = out_f32 && n_store <= 16 && cout == 64;
+    // the two kernels of 8 x 16 pixel tiles: bf16 results of all channels, or the head
+    const bool slopes = epi == cnok::EPI_SLOPE;
+    const bool head = out_f32 && n_store <= 16 && cout == 64 && !slopes;
     const bool plain = !out_f32 && n_store == cout && out_cs == cout;
-    if (cin == 64 && bn == 64 && (head || plain) && (epi != cnok::EPI_SLOPE || !((uintptr_t)slope_src & 15))) {
+    const cnok::ConvForm form = {n, h, w, cin, cout, slopes, head};
+    const long long halo = cnok::halo_tiles(form);
+    if ((head || plain) && halo <= 0x7fffffffLL && !(slopes && ((uintptr_t)slope_src & 15))) {
         cnok::ConvArgs b = a;
         b.tiles_w = (w + cnok::C64_W - 1) / cnok::C64_W;
         b.tiles_h = (h + cnok::C64_H - 1) / cnok::C64_H;
-        const long long t64 = (long long)n * b.tiles_w * b.tiles_h;
-        if (t64 <= HALO_TILES * tiles && t64 <= 0x7fffffffLL) {
-            b.tiles = (int)t64;
-            if (head)
-                return launch_conv64<16, false>(in, wmat, nullptr, b, st);
-            if (epi == cnok::EPI_SLOPE)
-                return launch_conv64<64, true>(in, wmat, slope_src, b, st);
-            return launch_conv64<64, false>(in, wmat, nullptr, b, st);
-        }
-    }
-    if (plain && cin <= 128 && cout % 128 == 0 && (epi != cnok::EPI_SLOPE || !((uintptr_t)slope_src & 15))) {
-        cnok::ConvArgs b = a;
-        b.tiles_w = (w + cnok::C64_W - 1) / cnok::C64_W;
-        b.tiles_h = (h + cnok::C64_H - 1) / cnok::C64_H;
-        const long long th = (long long)n * b.tiles_w * b.tiles_h;
-        if (th <= HALO_TILES * tiles && th <= 0x7fffffffLL) {
-            b.tiles = (int)th;
+        b.tiles = (int)halo;
+        const cnok::ConvKernel kernel = cnok::choose_conv(form, num_sms());
+        if (kernel == cnok::CONV_64)
+            return head     ? launch_conv64<16, false>(in, wmat, nullptr, b, st)
+                   : slopes ? launch_conv64<64, true>(in, wmat, slope_src, b, st)
+                            : launch_conv64<64, false>(in, wmat, nullptr, b, st);
+        if (kernel == cnok::CONV_HALO)
             return cin == 64 ? conv_halo<1>(in, wmat, slope_src, b, st) : conv_halo<2>(in, wmat, slope_src, b, st);
-        }
     }
     CUtensorMap mx, mw;
     CS(map_nhwc(&mx, in, n, h, w, cin, wt, ht));
