@@ -16,6 +16,7 @@
 #include "cno.h"
 #include "cno_dispatch.hpp"
 #include "cno_kernels.cuh"
+#include "per_device.hpp"
 
 using cnok::bf16;
 
@@ -172,6 +173,13 @@ static cudaError_t launch(void (*kern)(P...), dim3 grid, unsigned threads, size_
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
+// Opt-in of a kernel to more than 48 KB of dynamic shared memory (per device).
+template <class K>
+static cudaError_t allow_smem(K *kern, size_t bytes)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 static bool chan_ok(int c) { return c >= 64 && c % 64 == 0 && c <= 4096; }
 
 static cno_status check_image(int n, int h, int w)
@@ -199,11 +207,8 @@ static cno_status launch_fprop_bn(const CUtensorMap &mx, const CUtensorMap &mw, 
                                   cudaStream_t st)
 {
     using S = cnok::ConvShape<BN>;
-    static bool attr = false;
-    if (!attr) {
-        CK(cudaFuncSetAttribute(cnok::conv_fprop_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
-        attr = true;
-    }
+    static PerDevice ready;
+    CK(ready.once([] { return allow_smem(cnok::conv_fprop_kernel<BN>, S::SMEM); }));
     // persistent: at most the CTAs that fit on the SMs at once
     const int ctas = std::min(tiles, S::CTAS_PER_SM * num_sms());
     dim3 grid(ctas, a.cout / BN);
@@ -216,11 +221,8 @@ static cno_status launch_conv64(const void *in, const void *wmat, const void *sl
                                 cudaStream_t st)
 {
     using S = cnok::Conv64Shape<BN, SLOPE>;
-    static bool attr = false;
-    if (!attr) {
-        CK(cudaFuncSetAttribute(cnok::conv64_kernel<BN, SLOPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
-        attr = true;
-    }
+    static PerDevice ready;
+    CK(ready.once([] { return allow_smem(cnok::conv64_kernel<BN, SLOPE>, S::SMEM); }));
     CUtensorMap mx, mw, mo, ms;
     CS(map_nhwc(&mx, in, a.n, a.h, a.w, 64, cnok::C64_HW, cnok::C64_HH));
     CS(map_matrix(&mw, wmat, a.cout, 9 * 64, BN));
@@ -240,12 +242,8 @@ static cno_status launch_conv_halo(const void *in, const void *wmat, const void 
                                    cudaStream_t st)
 {
     using S = cnok::ConvHaloShape<CB>;
-    static bool attr = false;
-    if (!attr) {
-        CK(cudaFuncSetAttribute(cnok::conv_halo_kernel<CB, SLOPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                S::SMEM));
-        attr = true;
-    }
+    static PerDevice ready;
+    CK(ready.once([] { return allow_smem(cnok::conv_halo_kernel<CB, SLOPE>, S::SMEM); }));
     CUtensorMap mx, mw, mo, ms;
     CS(map_nhwc(&mx, in, a.n, a.h, a.w, a.cin, cnok::C64_HW, cnok::C64_HH));
     CS(map_matrix(&mw, wmat, a.cout, 9 * a.cin, S::BN));
@@ -349,11 +347,8 @@ static cno_status launch_wgrad_bn(const CUtensorMap &mdz, const CUtensorMap &mx,
                                   cudaStream_t st)
 {
     using S = cnok::WgradShape<BN>;
-    static bool attr = false;
-    if (!attr) {
-        CK(cudaFuncSetAttribute(cnok::conv_wgrad_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
-        attr = true;
-    }
+    static PerDevice ready;
+    CK(ready.once([] { return allow_smem(cnok::conv_wgrad_kernel<BN>, S::SMEM); }));
     dim3 grid(9 * a.mtiles * a.ntiles, a.splits);
     CK(launch(cnok::conv_wgrad_kernel<BN>, grid, 192, S::SMEM, st, mdz, mx, a));
     return CNO_OK;
@@ -364,11 +359,8 @@ static cno_status launch_wgrad64(const CUtensorMap &mdz, const CUtensorMap &mx, 
                                  cudaStream_t st)
 {
     using S = cnok::Wgrad64Shape<G>;
-    static bool attr = false;
-    if (!attr) {
-        CK(cudaFuncSetAttribute(cnok::wgrad64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
-        attr = true;
-    }
+    static PerDevice ready;
+    CK(ready.once([] { return allow_smem(cnok::wgrad64_kernel<G>, S::SMEM); }));
     CK(launch(cnok::wgrad64_kernel<G>, dim3(3 * (a.cout / 64), a.splits), 192, S::SMEM, st, mdz, mx, a));
     return CNO_OK;
 }

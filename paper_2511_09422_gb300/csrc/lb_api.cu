@@ -15,6 +15,7 @@
 
 #include "lb_kernels.cuh"
 #include "lbfreeze.h"
+#include "per_device.hpp"
 
 using lbk::Consts;
 
@@ -283,17 +284,25 @@ static cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, dim3 bloc
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
+// Attributes of a sweep: rings above 48 KB need the opt-in, and the carveout holds
+// every resident block.
+template <class K>
+static cudaError_t prepare(K *kern, int blocks, size_t smem)
+{
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_for(blocks, smem));
+}
+
 template <int MODE, class PS>
 static void launch_strip_as(const Consts &K, const lbk::Buffers &B, cudaStream_t st, double *partials)
 {
     constexpr size_t smem = lbk::strip_smem<PS, MODE != lbk::MODE_REDUCE>();
-    static bool opted = false;  // per instantiation: rings above 48 KB need the opt-in, and the
-    if (!opted) {               // carveout holds every resident block
-        cudaFuncSetAttribute(lbk::lb_strip_kernel<MODE, PS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(lbk::lb_strip_kernel<MODE, PS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             carveout_for(lbk::strip_min_blocks<PS, MODE != lbk::MODE_REDUCE>(), smem));
-        opted = true;
-    }
+    static PerDevice ready;
+    if (ready.once([] {
+            return prepare(lbk::lb_strip_kernel<MODE, PS>, lbk::strip_min_blocks<PS, MODE != lbk::MODE_REDUCE>(), smem);
+        }) != cudaSuccess)
+        return;  // the caller's cudaGetLastError reports it
     const unsigned grid = MODE == lbk::MODE_REDUCE ? reduce_blocks<PS>(K) : strip_blocks(K);
     launch_dependent(lbk::lb_strip_kernel<MODE, PS>, grid, dim3(32, LB_SW, 1), smem, st, K, B, partials);
 }
@@ -338,13 +347,9 @@ static cudaError_t launch_step_as(const lbk::StepRec *rec, int ninst, long long 
 {
     constexpr size_t smem = lbk::step_smem<PS>();
     constexpr int sw = lbk::step_warps<PS>();
-    static bool opted = false;
-    if (!opted) {
-        cudaFuncSetAttribute(lbk::lb_step_kernel<PS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(lbk::lb_step_kernel<PS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             carveout_for(lbk::step_min_blocks<PS>(), smem));
-        opted = true;
-    }
+    static PerDevice ready;
+    const cudaError_t e = ready.once([] { return prepare(lbk::lb_step_kernel<PS>, lbk::step_min_blocks<PS>(), smem); });
+    if (e != cudaSuccess) return e;
     // one persistent wave: as many blocks per SM as the rings of PS allow
     const long long wave = 152LL * lbk::step_min_blocks<PS>(), need = (nitems + sw - 1) / sw;
     const unsigned grid = (unsigned)(need < wave ? (need < 1 ? 1 : need) : wave);
