@@ -6,6 +6,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -17,6 +18,7 @@
 #include "cno_dispatch.hpp"
 #include "cno_kernels.cuh"
 #include "per_device.hpp"
+#include "slot_pool.hpp"
 
 using cnok::bf16;
 
@@ -710,6 +712,38 @@ static cno_status ensure_buffers(cno_net *net, int n, int h, int w, bool trainin
     return CNO_OK;
 }
 
+// Scratch of one acceptance check: the blocks' partial sums on the device (64 KB) and
+// the result in mapped host memory, written by the last kernel.  A call holds a slot
+// until it has synchronised its stream, so an idle slot is not in use; the idle ones
+// (at most four a device) are freed with the last network.  Allocating and freeing
+// device memory and copying the result in every call took 170 us beside 30 us of kernels.
+constexpr int CHECK_BLOCKS_MAX = 4 * 256, CHECK_VALUES = 8, MAX_DEVICES = 64;
+struct CheckSlot {
+    double *part = nullptr, *out = nullptr;
+};
+static SlotPool<CheckSlot, 4, MAX_DEVICES> g_check_slots;
+
+static void check_slot_free(CheckSlot s)
+{
+    cudaFree(s.part);
+    cudaFreeHost(s.out);
+}
+
+static cno_status check_slot_take(int dev, CheckSlot *s)
+{
+    if (g_check_slots.take(dev, s))
+        return CNO_OK;
+    cudaError_t e = cudaMalloc((void **)&s->part, (size_t)CHECK_BLOCKS_MAX * CHECK_VALUES * sizeof(double));
+    if (e == cudaSuccess)
+        e = cudaHostAlloc((void **)&s->out, CHECK_VALUES * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess)
+        check_slot_free(*s);
+    CK(e);
+    return CNO_OK;
+}
+
+static std::atomic<int> g_nets{0};  // live networks
+
 extern "C" cno_status cno_create(int cin, const int widths[4], int cout, int nf, cno_net **out)
 {
     if (!widths || !out)
@@ -722,6 +756,7 @@ extern "C" cno_status cno_create(int cin, const int widths[4], int cout, int nf,
     if (!chan_ok(cin) || cin > 256 || !chan_ok(cout) || cout > 256 || nf < 1 || nf > 8 || nf > cout)
         return fail(CNO_ERR_INVALID_ARG, "cin, cout must be multiples of 64 up to 256; 1 <= nf <= 8");
     cno_net *net = new cno_net();
+    g_nets++;
     net->cin = cin;
     net->cout = cout;
     net->nf = nf;
@@ -788,6 +823,9 @@ extern "C" cno_status cno_destroy(cno_net *net)
         if (p)
             cudaFree(p);
     delete net;
+    if (--g_nets == 0)
+        for (const CheckSlot &s : g_check_slots.drain())
+            check_slot_free(s);
     return CNO_OK;
 }
 
@@ -1141,7 +1179,7 @@ __global__ void __launch_bounds__(256) apply_update_kernel(FieldPtrs src, FieldO
 // warps.  Where an operand or product is so large (DIRECT, infinities and NaN) or so
 // small (the gradient below 2^-40, rho H below 2^-80) that an FP32 product or its rounding
 // error would leave the range, the cell's term is evaluated and added in FP64.
-constexpr int NCHK = 8;
+constexpr int NCHK = CHECK_VALUES;
 constexpr float DIRECT = 1e12f;
 constexpr float GRAD2_MIN = 8.2718061e-25f, CAP_MIN = 8.6736174e-19f, HEAT_MIN = 8.2718061e-25f;  // 2^-80, 2^-60, 2^-80
 constexpr float LATENT_MIN = 9.0949470e-13f;                                                        // 2^-40
@@ -1402,57 +1440,6 @@ extern "C" cno_status cno_apply_update(const float *const *src, float *const *ds
     return CNO_OK;
 }
 
-// Scratch of one check: the blocks' partial sums on the device (39 KB) and the result
-// in mapped host memory, written by the last kernel.  A call holds a slot until it
-// has synchronised its stream, so a returned slot is idle and calls on several
-// threads and streams never share one; up to CHECK_SLOTS idle slots are kept per
-// device.  Allocating and freeing device memory and copying the result in every call
-// took 170 us beside 30 us of kernels.
-constexpr int CHECK_SLOTS = 4, CHECK_BLOCKS_MAX = 4 * 256;
-struct CheckSlot {
-    double *part = nullptr, *out = nullptr;
-};
-static std::mutex g_check_mu;
-static std::vector<CheckSlot> g_check_slots[64];
-
-static void check_slot_free(CheckSlot &s)
-{
-    cudaFree(s.part);
-    cudaFreeHost(s.out);
-    s = CheckSlot();
-}
-
-static cno_status check_slot_take(int dev, CheckSlot *s)
-{
-    {
-        std::lock_guard<std::mutex> lk(g_check_mu);
-        if (!g_check_slots[dev].empty()) {
-            *s = g_check_slots[dev].back();
-            g_check_slots[dev].pop_back();
-            return CNO_OK;
-        }
-    }
-    cudaError_t e = cudaMalloc((void **)&s->part, (size_t)CHECK_BLOCKS_MAX * NCHK * sizeof(double));
-    if (e == cudaSuccess)
-        e = cudaHostAlloc((void **)&s->out, NCHK * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable);
-    if (e != cudaSuccess)
-        check_slot_free(*s);
-    CK(e);
-    return CNO_OK;
-}
-
-static void check_slot_return(int dev, CheckSlot &s)
-{
-    {
-        std::lock_guard<std::mutex> lk(g_check_mu);
-        if ((int)g_check_slots[dev].size() < CHECK_SLOTS) {
-            g_check_slots[dev].push_back(s);
-            return;
-        }
-    }
-    check_slot_free(s);
-}
-
 extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const float *T, const float *hcoef,
                                        int nx, int ny, double out[8], void *stream)
 {
@@ -1462,8 +1449,12 @@ extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const 
     const int blocks = std::min(std::min(ny, 4 * num_sms()), CHECK_BLOCKS_MAX);
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64)
+    if (dev < 0 || dev >= MAX_DEVICES)
         return fail(CNO_ERR_UNSUPPORTED, "device index out of range");
+    cudaStreamCaptureStatus capture;
+    CK(cudaStreamIsCapturing(st, &capture));
+    if (capture != cudaStreamCaptureStatusNone)
+        return fail(CNO_ERR_CUDA, "the checks wait for their result: not in a stream capture");
     HCoef hc = {0, 0, 0, 0, 0, 0};
     if (hcoef && fs && T) {
         hc = {hcoef[0], hcoef[1], hcoef[2], hcoef[3], 1, 0};
@@ -1483,10 +1474,8 @@ extern "C" cno_status cno_field_checks(const float *phi, const float *fs, const 
         e = se;
     if (e == cudaSuccess)
         memcpy(out, slot.out, NCHK * sizeof(double));
-    if (se == cudaSuccess)
-        check_slot_return(dev, slot);
-    else
-        check_slot_free(slot);  // the stream is in an error state
+    if (se != cudaSuccess || !g_check_slots.keep(dev, slot))
+        check_slot_free(slot);
     CK(e);
     if (!T)
         out[5] = out[6] = 0.0;
