@@ -14,7 +14,7 @@ CNO_LIB = os.path.join(PKG, "libcno.so")
 
 # (library, sources, headers it depends on)
 TARGETS = [
-    (LIB, ["lb_api.cu"], ["lb_kernels.cuh", "per_device.hpp", "lbfreeze.h"]),
+    (LIB, ["lb_api.cu"], ["lb_kernels.cuh", "per_device.hpp", "segment_rows.hpp", "lbfreeze.h"]),
     (CNO_LIB, ["cno_api.cu"], ["cno_kernels.cuh", "cno_dispatch.hpp", "per_device.hpp", "slot_pool.hpp", "cno.h"]),
 ]
 

@@ -16,6 +16,7 @@
 #include "lb_kernels.cuh"
 #include "lbfreeze.h"
 #include "per_device.hpp"
+#include "segment_rows.hpp"
 
 using lbk::Consts;
 
@@ -154,39 +155,15 @@ static std::string check_params(const lb_grid *g, const lb_params *p)
     return "";
 }
 
-// Rows of an inner segment: the height, at most max_rows, of the lowest estimated
-// step time when it cuts the work into items(h) items.  An item runs h + 3 rows
-// one after another (its own, and the fill of the rings).  The warps of the wave
-// take the items in rounds of W; a row takes longer the more warps share a
-// scheduler (1.45 us with one, 2.1 us with two FP32 warps; 1.6, 2.5 and 2.8 us with one, two
-// and three of a half form), and with many rounds the last one is only partly
-// filled.  Measured for heights 1 .. 16 (us per step):
-//   film 64 x 256: 9.2 at 2 rows, 17.0 at 8;   512 x 256: 15.1 at 4, 23.5 at 8;
-//   256^2: 11.4 at 2, 17.5 at 8;   512^2: 25.5 at 8, 28.5 at 4, 32.2 at 3;
-//   1037 x 771 (D2Q5): 61.6 at 12, 64.0 at 8, 72.2 at 10;   1024^2: 87.8 at 10, 95.1 at 12;
-//   F16: 512^2 26.6 at 6, 33.1 at 8, 29.9 at 3;   1024^2 76.7 at 16, 79.6 at 10, 87.1 at 8.
-// The estimate picks the best or the second best height in each of them.
+// Inner segment rows of a step: the height of the lowest estimated time when it cuts the
+// work into items(h) items (segment_rows.hpp).
 template <class Items>
-static int best_segment_rows(int kind, int max_rows, Items items)
+static int segment_rows_for(int kind, int max_rows, Items items)
 {
     const long long W = with_storage(kind, [](auto ps) {
         return 152LL * lbk::step_min_blocks<decltype(ps)>() * lbk::step_warps<decltype(ps)>();
     });
-    const bool half = kind == 1 || kind == 3;
-    int best = 1;
-    double least = 0.0;
-    for (int h = 1; h <= max_rows; h++) {
-        const long long n = items(h);
-        const double waves = (double)n / (double)W, rounds = waves <= 8.0 ? std::ceil(waves) : waves + 0.5;
-        const long long per_scheduler = ((n < W ? n : W) + 607) / 608;
-        const double share = per_scheduler <= 1 ? 1.0 : (!half ? 1.45 : (per_scheduler == 2 ? 1.55 : 1.75));
-        const double cost = rounds * (h + 3) * share;
-        if (h == 1 || cost < least) {
-            least = cost;
-            best = h;
-        }
-    }
-    return best;
+    return lbk::best_segment_rows(W, kind == 1 || kind == 3, max_rows, items);
 }
 
 static Consts make_consts(const lb_grid *g, const lb_params *p)
@@ -231,8 +208,9 @@ static Consts make_consts(const lb_grid *g, const lb_params *p)
     {
         const int kind = kind_of(p);
         const long long nstrip = (g->nx + LB_TX - 1) / LB_TX;
-        K.segh = best_segment_rows(kind, kind == 0 ? LB_SEGH : LB_SEGH_ALT,
-                                   [&](int h) { return nstrip * lbk::strip_segments(g->ny, h); });
+        const bool ragged = (kind == 1 || kind == 3) && g->nx % 8 != 0;
+        K.segh = segment_rows_for(kind, kind == 0 ? LB_SEGH : (ragged ? lbk::RAGGED_ROWS : LB_SEGH_ALT),
+                                  [&](int h) { return nstrip * lbk::strip_segments(g->ny, h); });
     }
     K.qfl = p->lattice_fl == LB_LATTICE_D2Q5 ? 5 : 9;
     K.divu = p->divu_mode;
@@ -983,7 +961,7 @@ extern "C" lb_status lb_batch_create(int n, const lb_grid *grids, const lb_param
         }
     }
     // the instances share the wave: segment heights for the work of the whole batch
-    const int segh = best_segment_rows(b->h[0]->kind, LB_SEGH_BATCH, [&](int rows) {
+    const int segh = segment_rows_for(b->h[0]->kind, LB_SEGH_BATCH, [&](int rows) {
         long long items = 0;
         for (const lb_handle *h : b->h)
             items += (long long)((h->K.nx + LB_TX - 1) / LB_TX) * lbk::strip_segments(h->K.ny, rows);
