@@ -962,10 +962,9 @@ extern "C" lb_status lb_batch_create(int n, const lb_grid *grids, const lb_param
     }
     // the instances share the wave: segment heights for the work of the whole batch
     const int segh = segment_rows_for(b->h[0]->kind, LB_SEGH_BATCH, [&](int rows) {
-        long long items = 0;
-        for (const lb_handle *h : b->h)
-            items += (long long)((h->K.nx + LB_TX - 1) / LB_TX) * lbk::strip_segments(h->K.ny, rows);
-        return items;
+        return lbk::batch_items(rows, [&](auto f) {
+            for (const lb_handle *h : b->h) f((h->K.nx + LB_TX - 1) / LB_TX, h->K.ny);
+        });
     });
     for (lb_handle *h : b->h) h->batch_segh = segh;
     b->inst.resize(n);
