@@ -102,6 +102,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
 }
 
 
+// A CTA in which a wait was given up may have loads under way into its shared memory and
+// MMAs that read it; it must not end before they are over.  Each role sets the abort
+// flag when it gives up, and then the issuing threads wait for what they issued, by
+// time alone (the status is set by then).  A CTA that ran to its end has seen the
+// end of both: the MMAs waited for every load, and the epilogue for every MMA.
+__device__ __noinline__ void mbar_drain(uint64_t *bar, uint32_t parity)
+{
+    if (mbar_try_wait(bar, parity))
+        return;
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(bar, parity) && global_ns() - t0 < WAIT_NS) {
+    }
+}
+// The last load of each slot of a ring whose slots were filled `fills` times in turn.
+template <int SLOTS>
+__device__ __forceinline__ void drain_loads(uint64_t *full, int fills)
+{
+    for (int s = 0; s < SLOTS && s < fills; s++)
+        mbar_drain(&full[s], ((fills - 1 - s) / SLOTS) & 1);
+}
+
 __device__ __forceinline__ void fence_barrier_init()
 {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -180,6 +201,13 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+
+// All MMAs that this thread has issued (bar: used for nothing else).
+__device__ __forceinline__ void drain_mmas(uint64_t *bar)
+{
+    umma_commit(bar);
+    mbar_drain(bar, 0);
 }
 
 // 32 consecutive FP32 columns of the warp's 32 tensor-memory lanes.
@@ -291,7 +319,8 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
     uint64_t *empty = full + S::STAGES;
     uint64_t *acc_full = empty + S::STAGES;  // [2]: the MMAs of a tile are done
     uint64_t *acc_empty = acc_full + 2;      // [2]: the epilogue has read the accumulator
-    uint32_t *tmem_holder = (uint32_t *)(acc_empty + 2);
+    uint64_t *drained = acc_empty + 2;
+    uint32_t *tmem_holder = (uint32_t *)(drained + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
     float *sbias = (float *)(smem + S::STAGES * S::STAGE + S::BAR_BYTES);
 
@@ -312,6 +341,7 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 4);  // one arrival per epilogue warp
         }
+        mbar_init(drained, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -324,10 +354,10 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    uint32_t loads = 0;  // stages filled by this thread
 
     if (warp == 0 && lane == 0) {
         // producer: the stage ring runs on across tiles
-        uint32_t kc = 0;
         for (int tile = blockIdx.x; tile < a.tiles && !*abort_flag; tile += gridDim.x) {
             int t = tile;
             const int tw = t % a.tiles_w;
@@ -336,9 +366,9 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
             const int img = t / a.tiles_h;
             const int w0 = tw * a.wt, h0 = th * a.ht;
             int cb = 0, dx = -1, dy = -1;  // channel block and tap of kb
-            for (int kb = 0; kb < a.kblocks; kb++, kc++) {
-                const int s = kc % S::STAGES;
-                const uint32_t use = kc / S::STAGES;
+            for (int kb = 0; kb < a.kblocks; kb++, loads++) {
+                const int s = loads % S::STAGES;
+                const uint32_t use = loads / S::STAGES;
                 if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1, a.status)) {
                     atomicOr(a.status, ST_TIMEOUT_PRODUCER);
                     *abort_flag = 1;
@@ -406,8 +436,10 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
             // the tensor-memory loads are warp-collective: take the decision per warp
             const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[acc], use & 1, a.status));
             if (!ok) {
-                if (lane == 0)
+                if (lane == 0) {
                     atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                    *abort_flag = 1;
+                }
                 break;
             }
             tc_fence_after();
@@ -495,6 +527,14 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
     }
     tc_fence_before();
     __syncthreads();
+    if (__builtin_expect(*abort_flag, 0)) {
+        if (warp == 0 && lane == 0) {
+            drain_loads<S::STAGES>(full, loads);
+        } else if (warp == 1 && lane == 0) {
+            drain_mmas(drained);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, S::TMEM_COLS);
@@ -578,7 +618,8 @@ __global__ void __launch_bounds__(192, 1)
     uint64_t *acc_empty = acc_full + 2; // [2]
     uint64_t *sl_full = acc_empty + 2;  // [2]
     uint64_t *sl_empty = sl_full + 2;   // [2]
-    uint32_t *tmem_holder = (uint32_t *)(sl_empty + 2);
+    uint64_t *drained = sl_empty + 2;
+    uint32_t *tmem_holder = (uint32_t *)(drained + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
     float *sbias = (float *)(smem + S::OFF_BAR + 256);
 
@@ -602,6 +643,7 @@ __global__ void __launch_bounds__(192, 1)
             mbar_init(&sl_full[b], 1);
             mbar_init(&sl_empty[b], 4);
         }
+        mbar_init(drained, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -614,6 +656,7 @@ __global__ void __launch_bounds__(192, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    int loads = 0, slopes = 0;  // tiles and slopes loaded by this thread
 
     auto place = [&](int tile, int &w0, int &h0, int &img) {
         const int tw = tile % a.tiles_w, r = tile / a.tiles_w;
@@ -636,6 +679,7 @@ __global__ void __launch_bounds__(192, 1)
                 *abort_flag = 1;
                 break;
             }
+            loads = it + 1;
             mbar_expect_tx(&full[s], S::A_BYTES);
             tma_load_4d(smem + S::OFF_A + s * S::A_STAGE, &map_x, &full[s], 0, w0 - 1, h0 - 1, img);
             if (SLOPE) {
@@ -645,6 +689,7 @@ __global__ void __launch_bounds__(192, 1)
                     *abort_flag = 1;
                     break;
                 }
+                slopes = it + 1;
                 mbar_expect_tx(&sl_full[b], S::TILE_BYTES);
                 tma_load_4d(smem + S::OFF_SLOPE + b * S::TILE_BYTES, &map_slope, &sl_full[b], n0, w0, h0, img);
             }
@@ -691,8 +736,10 @@ __global__ void __launch_bounds__(192, 1)
             if (SLOPE)
                 ok = ok && mbar_wait(&sl_full[acc], use & 1, a.status);
             if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0)
+                if (lane == 0) {
                     atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                    *abort_flag = 1;
+                }
                 break;
             }
             tc_fence_after();
@@ -785,6 +832,16 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (__builtin_expect(*abort_flag, 0)) {
+        if (warp == 0 && lane == 0) {
+            mbar_drain(w_full, 0);
+            drain_loads<S::STAGES>(full, loads);
+            drain_loads<2>(sl_full, slopes);
+        } else if (warp == 1 && lane == 0) {
+            drain_mmas(drained);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, S::TMEM_COLS);
@@ -843,7 +900,8 @@ __global__ void __launch_bounds__(224, 1)
     uint64_t *acc_full = b_empty + S::B_STAGES;          // [2]
     uint64_t *acc_empty = acc_full + 2;                  // [2]
     uint64_t *sl_full = acc_empty + 2;                   // [4 warps][2]
-    uint32_t *tmem_holder = (uint32_t *)(sl_full + 8);
+    uint64_t *drained = sl_full + 8;
+    uint32_t *tmem_holder = (uint32_t *)(drained + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
     float *sbias = (float *)(smem + S::OFF_BAR + 256);
 
@@ -868,6 +926,7 @@ __global__ void __launch_bounds__(224, 1)
         }
         for (int k = 0; k < 8; k++)
             mbar_init(&sl_full[k], 1);
+        mbar_init(drained, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -880,6 +939,7 @@ __global__ void __launch_bounds__(224, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    int loads = 0;  // tiles, weight stages or slopes loaded by this thread
 
     auto place = [&](int tile, int &w0, int &h0, int &img) {
         const int tw = tile % a.tiles_w, r = tile / a.tiles_w;
@@ -900,6 +960,7 @@ __global__ void __launch_bounds__(224, 1)
             }
             int w0, h0, img;
             place(tile, w0, h0, img);
+            loads = it + 1;
             mbar_expect_tx(&a_full[b], CB * S::A_BYTES);
             for (int c = 0; c < CB; c++)
                 tma_load_4d(smem + (b * CB + c) * S::A_BLOCK, &map_x, &a_full[b], c * KB, w0 - 1, h0 - 1, img);
@@ -913,6 +974,7 @@ __global__ void __launch_bounds__(224, 1)
                     *abort_flag = 1;
                     break;
                 }
+                loads++;
                 mbar_expect_tx(&b_full[s], S::G * S::B_BLOCK);
 #pragma unroll
                 for (int g = 0; g < S::G; g++)
@@ -982,6 +1044,7 @@ __global__ void __launch_bounds__(224, 1)
 #pragma unroll
                 for (int hf = 0; hf < BN / 64; hf++) {
                     uint64_t *bar = &sl_full[2 * q + ((it * (BN / 64) + hf) & 1)];
+                    loads++;
                     mbar_expect_tx(bar, 32 * ROW_BYTES);
                     tma_load_4d(stage(hf), &map_slope, bar, n0 + 64 * hf, w0, h0 + 4 * q, img);
                 }
@@ -995,8 +1058,10 @@ __global__ void __launch_bounds__(224, 1)
                     ok = ok && mbar_wait(&sl_full[2 * q + (u & 1)], (u >> 1) & 1, a.status);
                 }
             if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0)
+                if (lane == 0) {
                     atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                    *abort_flag = 1;
+                }
                 break;
             }
             tc_fence_after();
@@ -1056,6 +1121,19 @@ __global__ void __launch_bounds__(224, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (__builtin_expect(*abort_flag, 0)) {
+        if (lane == 0) {
+            if (warp == 0)
+                drain_loads<S::B_STAGES>(b_full, loads);
+            else if (warp == 1)
+                drain_mmas(drained);
+            else if (warp == 6)
+                drain_loads<S::A_BUFS>(a_full, loads);
+            else
+                drain_loads<2>(sl_full + 2 * (warp & 3), loads);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, S::TMEM_COLS);
@@ -1101,7 +1179,8 @@ __global__ void __launch_bounds__(192, 1)
     uint64_t *full = (uint64_t *)(smem + S::STAGES * S::STAGE);
     uint64_t *empty = full + S::STAGES;
     uint64_t *done = empty + S::STAGES;
-    uint32_t *tmem_holder = (uint32_t *)(done + 1);
+    uint64_t *drained = done + 1;
+    uint32_t *tmem_holder = (uint32_t *)(drained + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
 
     grid_begin();
@@ -1136,6 +1215,7 @@ __global__ void __launch_bounds__(192, 1)
             mbar_init(&empty[s], 1);
         }
         mbar_init(done, 1);
+        mbar_init(drained, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -1146,6 +1226,7 @@ __global__ void __launch_bounds__(192, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
     const int nk = kb_hi - kb_lo;
+    int loads = 0;  // stages filled by this thread
 
     if (warp == 0 && lane == 0) {
         const uint32_t bytes = (two_m ? 2 : 1) * SUB_BYTES + S::B_BYTES;
@@ -1160,6 +1241,7 @@ __global__ void __launch_bounds__(192, 1)
             }
             const int pw = tw * a.wt, ph = th * a.ht;
             uint8_t *st = smem + s * S::STAGE;
+            loads = j + 1;
             mbar_expect_tx(&full[s], bytes);
             tma_load_4d(st, &map_dz, &full[s], m0, pw, ph, img);
             if (two_m)
@@ -1212,8 +1294,10 @@ __global__ void __launch_bounds__(192, 1)
                 for (int c = 0; c < BN; c++)
                     dst[c] = 0.0f;
         } else if (!__all_sync(0xffffffffu, mbar_wait(done, 0, a.status))) {
-            if (lane == 0)
+            if (lane == 0) {
                 atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                *abort_flag = 1;
+            }
         } else {
             tc_fence_after();
             for (int c0 = 0; c0 < BN; c0 += 32) {
@@ -1229,6 +1313,14 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (__builtin_expect(*abort_flag, 0)) {
+        if (warp == 0 && lane == 0) {
+            drain_loads<S::STAGES>(full, loads);
+        } else if (warp == 1 && lane == 0) {
+            drain_mmas(drained);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, S::TMEM_COLS);
@@ -1275,7 +1367,8 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
     uint64_t *full = (uint64_t *)(smem + S::STAGES * S::STAGE);
     uint64_t *empty = full + S::STAGES;
     uint64_t *done = empty + S::STAGES;
-    uint32_t *tmem_holder = (uint32_t *)(done + 1);
+    uint64_t *drained = done + 1;
+    uint32_t *tmem_holder = (uint32_t *)(drained + 1);
     volatile int *abort_flag = (volatile int *)(tmem_holder + 1);
 
     grid_begin();
@@ -1294,6 +1387,7 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
             mbar_init(&empty[s], 1);
         }
         mbar_init(done, 1);
+        mbar_init(drained, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -1303,6 +1397,7 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    int loads = 0;  // stages filled by this thread
     const int pitch = (a.wt + 1) * ROW_BYTES;  // bytes of a staged image row
 
     // The two issuing threads keep their positions instead of dividing for them (which
@@ -1319,6 +1414,7 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
             }
             uint8_t *st = smem + s * S::STAGE;
             const int blocks = min(G, nk - j);
+            loads++;
             mbar_expect_tx(&full[s], blocks * bytes);
             for (int g = 0; g < blocks; g++, st += S::BLOCK) {
                 const int pw = tw * a.wt, ph = th * a.ht;
@@ -1382,8 +1478,10 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
         const bool have = nk > 0;
         const bool ok = !have || __all_sync(0xffffffffu, mbar_wait(done, 0, a.status));
         if (!ok) {
-            if (lane == 0)
+            if (lane == 0) {
                 atomicOr(a.status, ST_TIMEOUT_EPILOGUE);
+                *abort_flag = 1;
+            }
         } else {
             tc_fence_after();
 #pragma unroll 1
@@ -1404,6 +1502,14 @@ __global__ void __launch_bounds__(192, G == 4 ? 1 : 2)
     }
     tc_fence_before();
     __syncthreads();
+    if (__builtin_expect(*abort_flag, 0)) {
+        if (warp == 0 && lane == 0) {
+            drain_loads<S::STAGES>(full, loads);
+        } else if (warp == 1 && lane == 0) {
+            drain_mmas(drained);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, S::TMEM_COLS);
