@@ -151,8 +151,9 @@ cno_status cno_apply_update(const float *const *src, float *const *dst, int nfie
                             const float *out, int out_cs, const float *scale, const float *lo, const float *hi,
                             float phi_band, void *stream);
 
-/* Acceptance checks of a predicted state, FP64 sums in a fixed order over a
- * lattice with walls at y = 0 and y = ny - 1 and periodic x:
+/* Acceptance checks of a predicted state, sums to FP64's accuracy in a fixed
+ * order (terms as exact FP32 expansions, or in FP64) over a lattice with walls
+ * at y = 0 and y = ny - 1 and periodic x:
  *   out[0] = sum phi,  out[1] = sum chi, chi = clamp((1 + phi) / 2, 0, 1),
  *   out[2] = sum f_s (0 if fs is NULL),
  *   out[3] = sum (1 - phi^2),  out[4] = sum |grad phi| (central differences,
@@ -165,7 +166,7 @@ cno_status cno_apply_update(const float *const *src, float *const *dst, int nfie
  *   (0 if hcoef, fs or T is NULL).
  * The mass of the phase-change material is rho_s out[2] + rho_l (out[1] - out[2]);
  * for a flat profile phi = tanh(2 d / W) the width is W = 2 out[3] / out[4].
- * Synchronises the stream; out is host memory. */
+ * Synchronises the stream, which must not be in a capture; out is host memory. */
 cno_status cno_field_checks(const float *phi, const float *fs, const float *T, const float *hcoef, int nx, int ny,
                             double out[8], void *stream);
 

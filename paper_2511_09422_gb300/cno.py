@@ -286,7 +286,7 @@ def apply_update(src, dst, out, scale, phi_band=0.0, lo=None, hi=None):
 
 def field_checks(phi, fs=None, T=None, hcoef=None):
     """(sum phi, sum chi, sum f_s, sum (1 - phi^2), sum |grad phi|, min T, max T,
-    sum rho H) in FP64 of device fields [ny,nx]; hcoef = ((rho Cp)_l, (rho Cp)_s,
+    sum rho H) to FP64's accuracy of device fields [ny,nx]; hcoef = ((rho Cp)_l, (rho Cp)_s,
     (rho Cp)_g, rho_l L) for the enthalpy sum."""
     ny, nx = phi.shape
     out = (C.c_double * 8)()

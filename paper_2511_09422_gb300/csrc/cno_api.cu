@@ -375,15 +375,18 @@ static unsigned grid_for(long long n, int block)
 }
 
 // Whether wgrad64_kernel takes a weight gradient: 64 input channels, and rows of
-// at least 8 pixels (an 8-row group of its operands lies in one image row).
+// at least 8 pixels (an 8-row group of its operands lies in one image row).  Against
+// conv_wgrad_kernel, us with db, 64 and 192 output channels: 8^2 7.8/7.4 and 9.0/8.1, 64^2 10.6/9.2
+// and 13.4/11.8, 256 x 64 x 8 31.3/24.4 and 58.3/41.8, 16 x 256^2 176/137 and 406/298.
 static bool use_wgrad64(int w, int cin) { return cin == 64 && w >= 8; }
 
 // Tiling of a weight gradient: 64-pixel K blocks (wt x ht pixels of one
 // image), 9 taps x output-channel tiles x input-channel tiles, and as many
 // pixel ranges ("splits") as fill one wave of two CTAs per SM, with at least
-// 8 K blocks each.  wgrad64_kernel keeps the same ranges with a third of the CTAs:
-// the tensor cores round their running sums towards zero, so the length of a range
-// is part of the result's accuracy (1.5 times the ranges moved dW by 2.4e-5).
+// 8 K blocks each.  wgrad64_kernel keeps the same ranges with a third of the CTAs, so that
+// its sums are those of conv_wgrad_kernel to less than 1e-6.  The tensor cores round their
+// running sums towards zero: more ranges would be more accurate (16 x 256^2, error
+// against FP64 3.65e-5 with these 33, 2.43e-5 with 49) and faster (140, 109 us with db).
 static void wgrad_plan(int n, int h, int w, int cin, int cout, cnok::WgradArgs *a, int *bn)
 {
     *bn = pick_bn(cin);
@@ -1176,8 +1179,9 @@ __global__ void __launch_bounds__(256) apply_update_kernel(FieldPtrs src, FieldO
 // the sum of rho H.  Evaluating and adding a cell's terms in FP64 took 114 us at
 // 1024^2.  Here they are formed and added as FP32 expansions (f3, in cno_kernels.cuh)
 // that keep more than FP64's bits, and FP64 is left for the sums of the blocks'
-// warps.  Where an operand or product is so large (DIRECT, infinities and NaN) or so
-// small (the gradient below 2^-40, rho H below 2^-80) that an FP32 product or its rounding
+// warps.  (Two floats wide, a check took 14 us less and was off by up to 2^-46.)
+// Where an operand or product is so large (DIRECT, infinities and NaN) or so small
+// (the gradient below 2^-40, rho H below 2^-80) that an FP32 product or its rounding
 // error would leave the range, the cell's term is evaluated and added in FP64.
 constexpr int NCHK = CHECK_VALUES;
 constexpr float DIRECT = 1e12f;

@@ -557,8 +557,8 @@ __global__ void __launch_bounds__(192, ConvShape<BN>::CTAS_PER_SM)
 //     come in by TMA: whole lines both ways, no masks.
 // One persistent CTA per SM: TMA warp, MMA warp, four epilogue warps, two
 // accumulators.  The taps are added in the same order as in conv_fprop_kernel, so
-// the results are the same bits.  BN = 16 serves the head, of whose 64 outputs at
-// most 16 are stored.
+// the results are the same bits.  BN = 16 serves the head of small images, of whose 64
+// outputs at most 16 are stored.
 // --------------------------------------------------------------------------
 constexpr int C64_W = 8, C64_H = 16;              // pixels of a tile
 constexpr int C64_HW = C64_W + 2, C64_HH = C64_H + 2;

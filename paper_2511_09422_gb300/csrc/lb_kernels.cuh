@@ -1806,6 +1806,8 @@ __device__ __forceinline__ void unstream_set(const Consts &K, const InitTile &t,
             if (S == SET_G && i != 0) v += R(3.0) * wgt(i) * (t.p[nt] - t.p[n]);
         }
         if (S == SET_F) {
+            // w phi rounded for i > 0, fused for i = 0, as the stored states always were: a half
+            // population moves by a whole 11-bit step where the last bit of v differs
             const real w = wfl_rt(K.qfl, i);
             v = i == 0 ? __fmaf_rn(-w, phi_here, v) : __fsub_rn(v, __fmul_rn(w, phi_here));
         }

@@ -7,8 +7,8 @@ namespace lbk {
 // Greatest height of a half-storage lattice whose rows are not whole chunks of 8 values:
 // its strips at the x ends are staged lane by lane, and the taller their segments, the
 // longer a step waits for the last of them.  F16 with FP32 h, without this limit -> with
-// it (us per step): 1037 x 771 80.8 -> 72.4, 859 x 1230 104.2 -> 89.1, 2274 x 926 174 -> 161,
-// 1500 x 1300 159.5 -> 154.1; lattices that take no more than 12 rows anyway are the same.
+// it (us per step): 1037 x 771 80.8 -> 72.4, 859 x 1230 104.2 -> 89.1, 2274 x 926 174 -> 162,
+// 1500 x 1300 159.5 -> 151.2; lattices that take no more than 12 rows anyway are the same.
 constexpr int RAGGED_ROWS = 12;
 
 // Work items of a batch of lattices at h rows a segment; each(f) calls f(strips, ny) for

@@ -8,7 +8,7 @@ batched sweep, and planar fronts advancing toward an insoluble impurity), on
 the GPU, with the library's own forward and backward kernels.
 
 A jump is accepted only if the predicted state passes two checks against the
-state it started from (both computed by ``cno.field_checks`` in FP64):
+state it started from (both computed by ``cno.field_checks`` to FP64's accuracy):
 
 * mass of the phase-change material, M = rho_s sum f_s + rho_l sum (chi - f_s),
   conserved by the method (Sec. 2.1: the density change on freezing is what
